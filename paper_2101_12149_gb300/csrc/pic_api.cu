@@ -231,7 +231,7 @@ void keys_changed(pic_ctx* c) {
 cudaError_t run_hist(pic_ctx* c) {
     cudaError_t e;
     if (c->count_state != 0 &&
-        (e = cudaMemsetAsync(c->count, 0, (size_t(c->g.C) + 1) * sizeof(int), c->stream)) != cudaSuccess)
+        (e = cudaMemsetAsync(c->count, 0, (size_t(c->g.K) + 1) * sizeof(int), c->stream)) != cudaSuccess)
         return e;
     return counted(c, "k_hist", 1, pic::launch_hist);
 }
@@ -316,7 +316,7 @@ cudaError_t enqueue_step(pic_ctx* c, bool with_sort, bool count_next) {
 // Particle count after a sort with open z: the removed ones went to the last bin.
 cudaError_t read_live_count(pic_ctx* c) {
     int live = 0;
-    cudaError_t e = cudaMemcpyAsync(&live, c->offsets + c->g.C, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    cudaError_t e = cudaMemcpyAsync(&live, c->offsets + c->g.K, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess) c->np = live;
     return e;
@@ -403,7 +403,7 @@ cudaError_t save_state(pic_ctx* c, const StateLayout& L, char* dst, StateMeta& m
     if ((e = cudaMemcpyAsync(dst, c->P[c->cur].a[0], L.part, cudaMemcpyDeviceToDevice, c->stream))) return e;
     if ((e = cudaMemcpyAsync(dst + L.part, c->F[0], 9 * size_t(L.C) * L.rs, cudaMemcpyDeviceToDevice, c->stream)))
         return e;
-    if ((e = cudaMemcpyAsync(dst + L.part + L.fields, c->offsets, (size_t(L.C) + 1) * sizeof(int),
+    if ((e = cudaMemcpyAsync(dst + L.part + L.fields, c->offsets, (size_t(c->g.K) + 1) * sizeof(int),
                              cudaMemcpyDeviceToDevice, c->stream)))
         return e;
     if ((e = cudaMemcpyAsync(dst + L.part + L.fields + L.offs, c->d_step, sizeof(long long),
@@ -422,7 +422,7 @@ cudaError_t restore_state(pic_ctx* c, const StateLayout& L, const char* src, con
     if ((e = cudaMemcpyAsync(c->P[m.cur].a[0], src, L.part, cudaMemcpyDeviceToDevice, c->stream))) return e;
     if ((e = cudaMemcpyAsync(c->F[0], src + L.part, 9 * size_t(L.C) * L.rs, cudaMemcpyDeviceToDevice, c->stream)))
         return e;
-    if ((e = cudaMemcpyAsync(c->offsets, src + L.part + L.fields, (size_t(L.C) + 1) * sizeof(int),
+    if ((e = cudaMemcpyAsync(c->offsets, src + L.part + L.fields, (size_t(c->g.K) + 1) * sizeof(int),
                              cudaMemcpyDeviceToDevice, c->stream)))
         return e;
     if ((e = cudaMemcpyAsync(c->d_step, src + L.part + L.fields + L.offs, sizeof(long long),
@@ -513,6 +513,48 @@ pic_status read_error_word(pic_ctx* c) {
     if (h & pic::ERRBIT_TIMEOUT) return fail(PIC_ERR_TIMEOUT, "a bounded device-side wait ran out");
     if (h & pic::ERRBIT_RANGE) return fail(PIC_ERR_STATE, "a particle cell key was out of range");
     return fail(PIC_ERR_PARTICLE, "a particle became non-finite or moved a cell or more in one step");
+}
+
+// Automatic tiles: 4 x 4 x 32 cells when they divide the grid (a warp's lanes
+// then walk one z-row of cells), else 8 x 8 x 8 when those do.  Any other grid
+// is covered by whichever of the two overhangs it less: a tile's work follows
+// its cells inside the grid, but its staging and flush are paid whole, and the
+// smaller tiles that would divide such a grid cost far more of both
+// (100 x 75 x 90, order 2, 4 a cell: tiles of 4 x 1 x 2 took 8260 us a step,
+// overhanging 4 x 4 x 32 tiles 572 us, 8 x 8 x 8 548 us).  Orders 2 and 3 ask
+// for 5 % fewer cells before they take 4 x 4 x 32 (150 x 150 x 148, order 3:
+// 3320 us against 3186 us at 5 % more cells); order 1 in FP32-mixed has a
+// halo-1 layout with two CTAs an SM for 4 x 4 x 32 only and takes it up to
+// 1.4 times the cells (the same grid at order 1, 2 a cell: 591 us against 807;
+// 90 x 70 x 81: 245 against 299).  Grids whose overhanging keys would not fit
+// 31 bits get the largest powers of two up to 8 that divide them.
+void auto_tile(const int32_t n[3], int order, int prec, int T[3]) {
+    auto set = [&](int a, int b, int c) { T[0] = a, T[1] = b, T[2] = c; };
+    auto keys = [&](int a, int b, int c) {
+        return int64_t((n[0] + a - 1) / a) * ((n[1] + b - 1) / b) * ((n[2] + c - 1) / c) * (a * b * c);
+    };
+    const int64_t C = int64_t(n[0]) * n[1] * n[2];
+    const int64_t row = keys(4, 4, 32), cube = keys(8, 8, 8);
+    if (row == C) return set(4, 4, 32);
+    if (cube == C) return set(8, 8, 8);
+    const bool halo1 = order == 1 && prec == PIC_FP32_MIXED;
+    const bool use_row = halo1 ? double(row) <= 1.4 * double(cube) : double(row) <= 0.95 * double(cube);
+    if ((use_row ? row : cube) < (int64_t(1) << 31) - 1) return use_row ? set(4, 4, 32) : set(8, 8, 8);
+    for (int a = 0; a < 3; ++a) {
+        T[a] = 8;
+        while (T[a] > 1 && n[a] % T[a] != 0) T[a] >>= 1;
+    }
+}
+
+// Slabs per tile (log2): while the tiles leave SMs without work, each is cut
+// in two along x (one CTA then runs half the particles; every slab stages and
+// flushes its own halo, so no further than one slab an SM: 32^3 at order 3,
+// 4 a cell, 64 tiles: 106 us a step whole, 84 us in 128 halves, and with 256
+// quarters on 152 SMs 110 us; 16^3, 8 tiles: 78 us whole, 55 us in 64).
+int slab_cut(const pic::Geom& g, int sms) {
+    int lS = 0;
+    while ((g.T[0] >> (lS + 1)) >= 1 && (g.ntiles << (lS + 1)) <= sms) ++lS;
+    return lS;
 }
 
 pic_status check_ctx(pic_ctx* c) {
@@ -630,27 +672,18 @@ pic_status pic_init_grid(const pic_grid_desc* desc, void* cuda_stream, pic_ctx**
         c->sms = 1;
     }
     pic::Geom& g = c->g;
-    // Tiles: 4 x 4 x 32 cells when the grid allows (a warp's lanes then walk
-    // one z-row of cells), else the largest powers of two up to 8 per axis.
     int T[3];
     const bool given = D.tile[0] > 0 || D.tile[1] > 0 || D.tile[2] > 0;
     if (!given) {
-        if (D.n[0] % 4 == 0 && D.n[1] % 4 == 0 && D.n[2] % 32 == 0) {
-            T[0] = 4, T[1] = 4, T[2] = 32;
-        } else {
-            for (int a = 0; a < 3; ++a) {
-                T[a] = 8;
-                while (T[a] > 1 && D.n[a] % T[a] != 0) T[a] >>= 1;
-            }
-        }
+        auto_tile(D.n, D.order, D.precision, T);
     } else {
         for (int a = 0; a < 3; ++a) T[a] = D.tile[a];
+        for (int a = 0; a < 3; ++a)
+            if (!is_pow2(T[a]) || D.n[a] % T[a] != 0) {
+                delete c;
+                return fail(PIC_ERR_ARG, "tile extents must be powers of two dividing the grid");
+            }
     }
-    for (int a = 0; a < 3; ++a)
-        if (!is_pow2(T[a]) || D.n[a] % T[a] != 0) {
-            delete c;
-            return fail(PIC_ERR_ARG, "tile extents must be powers of two dividing the grid");
-        }
     if (T[0] <= 8 && T[1] <= 8 && T[2] <= 8) c->layout = 0;
     else if (T[0] <= 4 && T[1] <= 4 && T[2] <= 32) c->layout = D.precision == PIC_FP32_MIXED && D.order == 1 ? 2 : 1;
     else {
@@ -663,11 +696,13 @@ pic_status pic_init_grid(const pic_grid_desc* desc, void* cuda_stream, pic_ctx**
         g.L[a] = D.n[a] * D.d[a];
         g.T[a] = T[a];
         g.lT[a] = ilog2(T[a]);
-        g.nt[a] = D.n[a] / T[a];
+        g.nt[a] = (D.n[a] + T[a] - 1) / T[a];
     }
     g.cpt = g.T[0] * g.T[1] * g.T[2];
     g.C = C;
     g.ntiles = int64_t(g.nt[0]) * g.nt[1] * g.nt[2];
+    g.K = g.ntiles * g.cpt;
+    pic::set_slabs(g, D.sort_every == 1 ? slab_cut(g, c->sms) : 0);
     g.kbase = 0;
     g.zopen = D.window_axis == 2 ? 1 : 0;
     c->window = D.window_axis == 2;
@@ -689,13 +724,14 @@ pic_status pic_init_grid(const pic_grid_desc* desc, void* cuda_stream, pic_ctx**
         if ((e = cudaMemset(fb, 0, 9 * C * c->rsize)) != cudaSuccess) return bail(e, "field zeroing");
     }
     if (c->Fo[0] && (e = pic::configure_yee_fused()) != cudaSuccess) return bail(e, "Yee kernel configuration");
-    // one bin more than cells (removed particles, open z) and its offset
-    if ((e = cudaMalloc(&c->count, (C + 1) * sizeof(int))) != cudaSuccess) return bail(e, "count allocation");
-    if ((e = cudaMemset(c->count, 0, (C + 1) * sizeof(int))) != cudaSuccess) return bail(e, "count zeroing");
-    if ((e = cudaMalloc(&c->offsets, (C + 2) * sizeof(int))) != cudaSuccess) return bail(e, "offsets allocation");
-    if ((e = cudaMemset(c->offsets, 0, (C + 2) * sizeof(int))) != cudaSuccess) return bail(e, "offsets zeroing");
-    c->scan_chunks = int(pic::scan_status_words(C + g.zopen) - 1);
-    if ((e = cudaMalloc(&c->scan_status, pic::scan_status_words(C + 1) * sizeof(unsigned long long))) != cudaSuccess)
+    // one bin more than cell keys (removed particles, open z) and its offset
+    const int64_t K = g.K;
+    if ((e = cudaMalloc(&c->count, (K + 1) * sizeof(int))) != cudaSuccess) return bail(e, "count allocation");
+    if ((e = cudaMemset(c->count, 0, (K + 1) * sizeof(int))) != cudaSuccess) return bail(e, "count zeroing");
+    if ((e = cudaMalloc(&c->offsets, (K + 2) * sizeof(int))) != cudaSuccess) return bail(e, "offsets allocation");
+    if ((e = cudaMemset(c->offsets, 0, (K + 2) * sizeof(int))) != cudaSuccess) return bail(e, "offsets zeroing");
+    c->scan_chunks = int(pic::scan_status_words(K + g.zopen) - 1);
+    if ((e = cudaMalloc(&c->scan_status, pic::scan_status_words(K + 1) * sizeof(unsigned long long))) != cudaSuccess)
         return bail(e, "scan state allocation");
     if ((e = cudaMalloc(&c->err, 8 * sizeof(unsigned))) != cudaSuccess) return bail(e, "error word allocation");
     if ((e = cudaMemset(c->err, 0, 8 * sizeof(unsigned))) != cudaSuccess) return bail(e, "error word");

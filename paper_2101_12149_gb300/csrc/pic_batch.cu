@@ -121,7 +121,9 @@ pic::Geom box_geom(const BoxInfo& B, const int tile[3]) {
     }
     g.cpt = g.T[0] * g.T[1] * g.T[2];
     g.C = C;
+    g.K = C;  // the tiles divide the box
     g.ntiles = int64_t(g.nt[0]) * g.nt[1] * g.nt[2];
+    pic::set_slabs(g, 0);
     g.kbase = int(B.cbase);
     g.zopen = 0;
     return g;
@@ -511,6 +513,7 @@ pic_status pic_batch_init(int32_t nboxes, const int32_t* n, const double* d, con
     P.order = 0;
     std::memset(&P.g, 0, sizeof(P.g));
     P.g.C = C;
+    P.g.K = C;
     for (auto& B : b->box) B.g = box_geom(B, b->tune.tile);
     auto bail = [&](cudaError_t e, const char* what) {
         pic_batch_destroy(b);

@@ -15,7 +15,7 @@ namespace pic {
 enum : unsigned {
     ERRBIT_PARTICLE = 1u,  // non-finite particle or a move of >= 1 cell
     ERRBIT_TIMEOUT = 2u,   // a bounded wait ran out
-    ERRBIT_RANGE = 4u,     // a sort key outside [0, C)
+    ERRBIT_RANGE = 4u,     // a sort key outside [0, K)
     ERRBIT_CHECK = 8u,     // a device-side self-check failed (see check word); most run in checking builds only
 };
 
@@ -38,18 +38,36 @@ struct Geom {
     int n[3];      // cells per axis
     int T[3];      // cells per tile per axis (powers of two)
     int lT[3];     // log2 T
-    int nt[3];     // tiles per axis
+    int nt[3];     // tiles per axis (the last one of an axis may overhang the grid)
     int cpt;       // cells per tile
     int64_t C;     // cells
+    int64_t K;     // cell keys: ntiles * cpt (more than C where the tiles overhang the grid)
     int64_t ntiles;
     double d[3];
     double L[3];
+    // The tile kernel's work items: each tile cut into 2^lS slabs of cells
+    // along x (contiguous key ranges, since x is the slowest axis inside a
+    // tile); W = cells per slab per axis, cpw cells a slab, nwork slabs.
+    int lS;
+    int W[3];
+    int cpw;
+    int64_t nwork;
     int kbase;     // added to every cell key (a box's first key in a batch of boxes; 0 otherwise)
     int zopen;     // 1: z is open (moving window): no field beyond the z ends, particles leaving z die
 };
 
-// Key of a removed particle: one past the last cell; the sort puts these last.
-__host__ __device__ inline int dead_key(const Geom& g) { return g.kbase + int(g.C); }
+// Key of a removed particle: one past the last cell key; the sort puts these last.
+__host__ __device__ inline int dead_key(const Geom& g) { return g.kbase + int(g.K); }
+
+// Cut the tiles of g into 2^lS slabs along x (2^lS <= T[0]).
+inline void set_slabs(Geom& g, int lS) {
+    g.lS = lS;
+    g.W[0] = g.T[0] >> lS;
+    g.W[1] = g.T[1];
+    g.W[2] = g.T[2];
+    g.cpw = g.cpt >> lS;
+    g.nwork = g.ntiles << lS;
+}
 
 struct Timer {
     const char* name;
@@ -102,14 +120,14 @@ struct pic_ctx {
     CUtensorMap tmap_eb_o;  // the other set's E/B
     bool tma_o = false;
 
-    int* count = nullptr;    // per-cell particle counts [C]
+    int* count = nullptr;    // per-cell particle counts [K]
     // What count holds: 0 all zero (a scatter leaves it so), 1 the histogram
     // of the current keys (a tile kernel counted its particles' new keys),
     // 2 stale (non-zero, not the current keys: cleared before the next
     // histogram).  count_into: the next tile-kernel launch counts.
     int count_state = 0;
     bool count_into = false;
-    int* offsets = nullptr;  // exclusive scan of count [C+1]; tile t owns [offsets[t*cpt], offsets[(t+1)*cpt])
+    int* offsets = nullptr;  // exclusive scan of count [K+1]; tile t owns [offsets[t*cpt], offsets[(t+1)*cpt])
     unsigned long long* scan_status = nullptr;  // look-back words + ticket
     int scan_chunks = 0;
     bool sorted = false;       // particles are in tile order of the current offsets
@@ -282,7 +300,7 @@ struct StateLayout {
         ints = align(cap * sizeof(int));
         part = 7 * per + 2 * ints;
         fields = align(9 * size_t(C) * rs);
-        offs = align((size_t(C) + 1) * sizeof(int));
+        offs = align((size_t(c->g.K) + 1) * sizeof(int));
         total = part + fields + offs + 256;
     }
     pic::Snapshot view(char* base) const {

@@ -442,7 +442,7 @@ __device__ __forceinline__ void flush_fixed4(const StepArgs<R>& A, int* sJi, int
     const int q4 = Q4c > 0 ? Q4c : q4_rt;
     const int per_c = jx * jy * q4;
     for (int e = threadIdx.x; e < 3 * per_c; e += blockDim.x) {
-        const int c = e / per_c;
+        const int c = int(e >= per_c) + int(e >= 2 * per_c);
         int r = e - c * per_c;
         const int row = r / q4;
         const int q = r - row * q4;
@@ -478,10 +478,10 @@ __device__ __forceinline__ void flush_tile(const StepArgs<R>& A, R* sJ, int oi, 
     const Geom& g = A.g;
     constexpr bool kFixed = sizeof(R) == 4;
     int* sJi = reinterpret_cast<int*>(sJ);
-    const int jx = g.T[0] + 2 * LY::H + 1, jy = g.T[1] + 2 * LY::H + 1, jz = g.T[2] + 8;
-    if (kFixed && (g.T[2] % 4) == 0 && (g.n[2] % 4) == 0) {
-        // the layout's own tile shape indexes the J box with constants
-        if (jx == LY::JX && jy == LY::JY && jz == LY::JZ)
+    const int jx = g.W[0] + 2 * LY::H + 1, jy = g.W[1] + 2 * LY::H + 1, jz = g.W[2] + 8;
+    if (kFixed && (g.W[2] % 4) == 0 && (g.n[2] % 4) == 0) {
+        // the layout's own y and z extents index the J box with constants
+        if (jy == LY::JY && jz == LY::JZ)
             flush_fixed4<R, LY, LY::JY, LY::JZ / 4>(A, sJi, oi, oj, ok, jx, jy, jz / 4);
         else
             flush_fixed4<R, LY, 0, 0>(A, sJi, oi, oj, ok, jx, jy, jz / 4);
@@ -489,7 +489,7 @@ __device__ __forceinline__ void flush_tile(const StepArgs<R>& A, R* sJ, int oi, 
     }
     const int vol = jx * jy * jz;
     for (int e = threadIdx.x; e < 3 * vol; e += blockDim.x) {
-        const int c = e / vol;
+        const int c = int(e >= vol) + int(e >= 2 * vol);
         int r = e - c * vol;
         const int a = r / (jy * jz);
         r -= a * jy * jz;
@@ -542,17 +542,17 @@ struct TileWork {
 template <typename R>
 __device__ __forceinline__ void plan_tile(const StepArgs<R>& A, int t, TileWork& w) {
     const Geom& g = A.g;
-    w.beg = A.offsets[(int64_t)t * g.cpt];
-    w.end = A.offsets[(int64_t)(t + 1) * g.cpt];
+    w.beg = A.offsets[(int64_t)t * g.cpw];
+    w.end = A.offsets[(int64_t)(t + 1) * g.cpw];
     const int cnt = w.end - w.beg;
     const int lane = threadIdx.x & 31;
     const int nwarp = blockDim.x >> 5;
     w.wbeg = w.beg;
     w.wend = w.end;
     bool by_warp = false;
-    if (A.run <= 0 && g.cpt % nwarp == 0 && nwarp <= 32) {
-        const int cpw = g.cpt / nwarp;
-        const int64_t c0 = (int64_t)t * g.cpt;
+    if (A.run <= 0 && g.cpw % nwarp == 0 && nwarp <= 32) {
+        const int cpw = g.cpw / nwarp;
+        const int64_t c0 = (int64_t)t * g.cpw;
         const int gsize =
             lane < nwarp ? A.offsets[c0 + (int64_t)(lane + 1) * cpw] - A.offsets[c0 + (int64_t)lane * cpw] : 0;
         const int gmax = __reduce_max_sync(0xffffffffu, gsize);
@@ -571,7 +571,7 @@ __device__ __forceinline__ void plan_tile(const StepArgs<R>& A, int t, TileWork&
         w.rstart = 0;
         w.rstride = 32;
     } else {
-        w.run = A.run > 0 ? A.run : max(1, (cnt + (g.cpt >> 1)) / g.cpt);
+        w.run = A.run > 0 ? A.run : max(1, (cnt + (g.cpw >> 1)) / g.cpw);
         w.nrun = (cnt + w.run - 1) / w.run;
         w.rstart = threadIdx.x - lane;
         w.rstride = blockDim.x;
@@ -605,8 +605,8 @@ __device__ __forceinline__ void decode_in_tile(const StepArgs<R>& A, const RawPa
         const Geom& g = A.g;
         const int kk = r.key - g.kbase;
         const int ls = g.lT[1] + g.lT[2];
-        if ((kk >> (g.lT[0] + ls)) == t) {
-            const int l = kk & (g.cpt - 1);
+        if ((kk >> (g.lT[0] - g.lS + ls)) == t) {
+            const int l = kk & (g.cpw - 1);
             cell[0] = oi + (l >> ls);
             cell[1] = oj + ((l >> g.lT[2]) & (g.T[1] - 1));
             cell[2] = ok + (l & (g.T[2] - 1));
@@ -660,8 +660,8 @@ __device__ __forceinline__ void tile_particles(const StepArgs<R>& A, const TileW
                 decode_in_tile<R>(A, raw, t, oi, oj, ok, cell, f0, xg0, u, wq);
                 const int li = cell[0] - oi, lj = cell[1] - oj, lk = cell[2] - ok;
                 // the fixed-point sums are exact for up to 65535 particles per tile
-                const bool inside = unsigned(li) < unsigned(g.T[0]) && unsigned(lj) < unsigned(g.T[1]) &&
-                                    unsigned(lk) < unsigned(g.T[2]) && (!kFixed || p - w.beg < 65535);
+                const bool inside = unsigned(li) < unsigned(g.W[0]) && unsigned(lj) < unsigned(g.W[1]) &&
+                                    unsigned(lk) < unsigned(g.W[2]) && (!kFixed || p - w.beg < 65535);
                 if (!inside) {
                     const int slot = atomicAdd(A.outn, 1);
                     A.outl[slot] = p;
@@ -748,7 +748,7 @@ template <typename R, class LY>
 __device__ __forceinline__ void restage_wrapped(const StepArgs<R>& A, R* sEB, int oi, int oj, int ok) {
     const Geom& g = A.g;
     constexpr int H = LY::H;
-    const int ex = g.T[0] + 2 * H, ey = g.T[1] + 2 * H, ez = g.T[2] + 2 * H;
+    const int ex = g.W[0] + 2 * H, ey = g.W[1] + 2 * H, ez = g.W[2] + 2 * H;
     if (oi < H) stage_box<R, LY>(A, sEB, oi, oj, ok, 0, H - oi, 0, ey, 0, ez);
     if (oi + ex - H > g.n[0]) stage_box<R, LY>(A, sEB, oi, oj, ok, g.n[0] - oi + H, ex, 0, ey, 0, ez);
     if (oj < H) stage_box<R, LY>(A, sEB, oi, oj, ok, 0, ex, 0, H - oj, 0, ez);
@@ -763,7 +763,7 @@ __device__ __forceinline__ void restage_wrapped(const StepArgs<R>& A, R* sEB, in
 template <typename R, class LY>
 __device__ __forceinline__ void stage_all(const StepArgs<R>& A, R* sEB, int oi, int oj, int ok) {
     const Geom& g = A.g;
-    const int ex = g.T[0] + 2 * LY::H, ey = g.T[1] + 2 * LY::H, ez = g.T[2] + 2 * LY::H;
+    const int ex = g.W[0] + 2 * LY::H, ey = g.W[1] + 2 * LY::H, ez = g.W[2] + 2 * LY::H;
     if (ex == LY::EX && ey == LY::EY && ez == LY::EZ)
         stage_box<R, LY, true>(A, sEB, oi, oj, ok, 0, ex, 0, ey, 0, ez);
     else
@@ -771,11 +771,11 @@ __device__ __forceinline__ void stage_all(const StepArgs<R>& A, R* sEB, int oi, 
 }
 
 // Next tile with particles from the queue (one thread), or -1 when none is left.
-__device__ __forceinline__ int next_tile(const int* __restrict__ offsets, int cpt, int ntiles, int* queue) {
+__device__ __forceinline__ int next_tile(const int* __restrict__ offsets, int cpw, int nwork, int* queue) {
     for (;;) {
         const int t = atomicAdd(queue, 1);
-        if (t >= ntiles) return -1;
-        if (offsets[(int64_t)(t + 1) * cpt] > offsets[(int64_t)t * cpt]) return t;
+        if (t >= nwork) return -1;
+        if (offsets[(int64_t)(t + 1) * cpw] > offsets[(int64_t)t * cpw]) return t;
     }
 }
 
@@ -794,14 +794,14 @@ __device__ __forceinline__ void tile_loop(const StepArgs<R>& A, int* queue, unsi
     constexpr int kZShift = tma_layout<LY, R>() ? 4 - LY::H : 0;
     R* sEB = sm + kZShift;
     R* sJ = sm + 6 * LY::eVol;
-    const int ntiles = int(g.ntiles);
+    const int nwork = int(g.nwork);
     __shared__ __align__(8) unsigned long long s_bar;
     __shared__ int s_tile[2];
 
     zero_jbox<R, LY>(sJ);
     if (threadIdx.x == 0) {
         mbar_init(&s_bar);
-        s_tile[0] = next_tile(A.offsets, g.cpt, ntiles, queue);
+        s_tile[0] = next_tile(A.offsets, g.cpw, nwork, queue);
     }
     __syncthreads();
     int t = s_tile[0];
@@ -810,7 +810,7 @@ __device__ __forceinline__ void tile_loop(const StepArgs<R>& A, int* queue, unsi
         return;
     }
     int oi, oj, ok;
-    tile_origin(g, t, oi, oj, ok);
+    work_origin(g, t, oi, oj, ok);
     TileWork w;
     plan_tile<R>(A, t, w);
     RawParticle<R> next;
@@ -824,7 +824,7 @@ __device__ __forceinline__ void tile_loop(const StepArgs<R>& A, int* queue, unsi
     }
     unsigned phase = 0;  // parity of the barrier phase the next TMA copy completes
     for (;;) {
-        if (threadIdx.x == 0) s_tile[1] = next_tile(A.offsets, g.cpt, ntiles, queue);
+        if (threadIdx.x == 0) s_tile[1] = next_tile(A.offsets, g.cpw, nwork, queue);
         if (by_tma) {
             // every thread waits for the copy; if it did not land in time, all
             // wait once more (it is still writing into this CTA's shared
@@ -848,7 +848,7 @@ __device__ __forceinline__ void tile_loop(const StepArgs<R>& A, int* queue, unsi
         int ni = 0, nj = 0, nk = 0;
         bool tma_n = false;
         if (tn >= 0) {
-            tile_origin(g, tn, ni, nj, nk);
+            work_origin(g, tn, ni, nj, nk);
             tma_n = tile_uses_tma<R, LY>(tmap, sm, nk);
             if (tma_n && threadIdx.x == 0)
                 tma_load_eb(tmap, sm, &s_bar, unsigned(6 * LY::eVol * sizeof(R)), nk - 4, nj - LY::H, ni - LY::H);
@@ -884,8 +884,8 @@ __device__ __forceinline__ int next_item(const StepArgs<R>* __restrict__ boxes, 
         if (it >= nitems) return -1;
         const int2 bt = items[it];
         const StepArgs<R>& B = boxes[bt.x];
-        const int cpt = B.g.cpt;
-        if (B.offsets[(int64_t)(bt.y + 1) * cpt] > B.offsets[(int64_t)bt.y * cpt]) return it;
+        const int cpw = B.g.cpw;
+        if (B.offsets[(int64_t)(bt.y + 1) * cpw] > B.offsets[(int64_t)bt.y * cpw]) return it;
     }
 }
 
@@ -929,7 +929,7 @@ __global__ void __launch_bounds__(LY::kThreads, LY::kMinBlocks)
     __syncthreads();
     int t = items[it].y;
     int oi, oj, ok;
-    tile_origin(sA[0].g, t, oi, oj, ok);
+    work_origin(sA[0].g, t, oi, oj, ok);
     TileWork w;
     plan_tile<R>(sA[0], t, w);
     RawParticle<R> next;
@@ -966,7 +966,7 @@ __global__ void __launch_bounds__(LY::kThreads, LY::kMinBlocks)
             const int2 bt = items[itn];
             const StepArgs<R>& An = boxes[bt.x];  // read from global until its slot is filled
             tn = bt.y;
-            tile_origin(An.g, tn, ni, nj, nk);
+            work_origin(An.g, tn, ni, nj, nk);
             tma_n = tile_uses_tma<R, LY>(An.tmap, sm, nk);
             if (tma_n && threadIdx.x == 0)
                 tma_load_eb(An.tmap, sm, &s_bar, unsigned(6 * LY::eVol * sizeof(R)), nk - 4, nj - LY::H, ni - LY::H);
@@ -1155,7 +1155,7 @@ static inline unsigned blocks_for(int64_t n) { return unsigned((n + kBlock - 1) 
 
 // Persistent CTAs of the tile kernel: as many as fit on the GPU at once (the
 // SM count times the CTAs per SM the kernel's resources allow), at most one
-// per tile.
+// per work item.
 template <typename R, int P, class LY> int tile_grid(const pic_ctx* c) {
     static int per_sm = 0;  // per instantiation; found outside stream capture by pic_init_grid
     if (per_sm == 0) {
@@ -1169,7 +1169,7 @@ template <typename R, int P, class LY> int tile_grid(const pic_ctx* c) {
         per_sm = n;
     }
     const int64_t g = int64_t(c->sms) * per_sm;
-    return int(g < c->g.ntiles ? g : c->g.ntiles);
+    return int(g < c->g.nwork ? g : c->g.nwork);
 }
 
 template <typename R, int P, class LY> cudaError_t tile_step_impl(pic_ctx* c) {

@@ -314,12 +314,13 @@ __global__ void __launch_bounds__(kSortBlock) k_bin_keys(const int* __restrict__
 
 size_t scan_status_words(int64_t C) { return size_t((C + kScanChunk - 1) / kScanChunk) + 1; }
 
-// Bins of the sort: one per cell, plus one for removed particles when z is
+// Bins of the sort: one per cell key, plus one for removed particles when z is
 // open; with pic_sort_particles' coarse bins one per run of 2^sort_shift
 // cells, with its random bins one per cell.
 static int64_t nbins(const pic_ctx* c) {
-    if (c->sort_shift > 0) return ((c->g.C - 1) >> c->sort_shift) + 1;
-    return c->g.C + (c->g.zopen ? 1 : 0);
+    if (c->sort_shift > 0) return ((c->g.K - 1) >> c->sort_shift) + 1;
+    if (c->sort_shift < 0) return c->g.C;
+    return c->g.K + (c->g.zopen ? 1 : 0);
 }
 static const int* bins(const pic_ctx* c) { return c->sort_shift == 0 ? c->P[c->cur].key : c->sortbin; }
 

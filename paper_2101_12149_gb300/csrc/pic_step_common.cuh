@@ -37,6 +37,12 @@ __device__ __forceinline__ void tile_origin(const Geom& g, int t, int& oi, int& 
     ok = tk << g.lT[2];
 }
 
+// First cell of work item w (slab w mod 2^lS of its tile).
+__device__ __forceinline__ void work_origin(const Geom& g, int w, int& oi, int& oj, int& ok) {
+    tile_origin(g, w >> g.lS, oi, oj, ok);
+    oi += (w & ((1 << g.lS) - 1)) * g.W[0];
+}
+
 __device__ __forceinline__ void cell_of(const Geom& g, int key, int& i, int& j, int& k) {
     key -= g.kbase;
     const int lcpt = g.lT[0] + g.lT[1] + g.lT[2];

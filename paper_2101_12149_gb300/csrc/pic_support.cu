@@ -752,6 +752,9 @@ template <typename R> cudaError_t yee_fused_impl(pic_ctx* c) {
     const int64_t want = 4 * int64_t(c->sms > 0 ? c->sms : 148) * (c->prec == PIC_FP64 ? 3 : 6);
     Y.xc = 32;
     while (Y.xc > 8 && tiles * ((c->g.n[0] + Y.xc - 1) / Y.xc) < want) Y.xc /= 2;
+    // a grid too small for one block an SM even so: shorter chunks, since a
+    // block's march of xc + 2 dependent steps is then the launch's whole time
+    while (Y.xc > 1 && tiles * ((c->g.n[0] + Y.xc - 1) / Y.xc) < (c->sms > 0 ? c->sms : 148)) Y.xc /= 2;
     Y.nt[0] = (c->g.n[0] + Y.xc - 1) / Y.xc;
     Y.h = R(0.5 * c->dt);
     Y.dt = R(c->dt);
