@@ -98,13 +98,24 @@ template <typename R> struct Shape<2, R> {
 template <typename R> struct Shape<3, R> {
     __device__ __forceinline__ static void weights(R f, int& first, R w[4]) {
         first = -1;
-        const R f2 = f * f, f3 = f2 * f;
-        const R g = R(1) - f;
         const R sixth = R(1) / R(6);
-        w[0] = g * g * g * sixth;
-        w[1] = (R(4) - R(6) * f2 + R(3) * f3) * sixth;
-        w[2] = (R(1) + R(3) * f + R(3) * f2 - R(3) * f3) * sixth;
-        w[3] = f3 * sixth;
+        const R f2 = f * f, g = R(1) - f;
+        if constexpr (sizeof(R) == 8) {
+            // the pieces are mirror images in f and g: 11 operations on the FP64
+            // pipe, which bounds that path, against 15 (in FP32 the rounding of
+            // 2/3 would raise the bias of the weights' sum from 3.0e-8 to 4.2e-8)
+            const R g2 = g * g, two_thirds = R(2) / R(3);
+            w[0] = g2 * g * sixth;
+            w[1] = two_thirds + f2 * (R(0.5) * f - R(1));
+            w[2] = two_thirds + g2 * (R(0.5) * g - R(1));
+            w[3] = f2 * f * sixth;
+        } else {
+            const R f3 = f2 * f;
+            w[0] = g * g * g * sixth;
+            w[1] = (R(4) - R(6) * f2 + R(3) * f3) * sixth;
+            w[2] = (R(1) + R(3) * f + R(3) * f2 - R(3) * f3) * sixth;
+            w[3] = f3 * sixth;
+        }
     }
 };
 
@@ -176,9 +187,17 @@ __device__ __forceinline__ void staggered_weights_ec(R f, int& first, R w[P + 1]
 // FP64: both half kicks, g-, t, s and the rotation, so its stored FP32
 // momentum is rounded once per step.
 // ---------------------------------------------------------------------------
+// 1 / sqrt(v).  FP64: the reciprocal square root itself (error within an ulp,
+// as of the square root and division it replaces) spends a third of their
+// operations on the FP64 pipe.
+__device__ __forceinline__ double inv_sqrt(double v) { return rsqrt(v); }
+__device__ __forceinline__ float inv_sqrt(float v) { return 1.0f / sqrtf(v); }
+
+// g2 = g-^2
 template <typename R>
-__device__ __forceinline__ void boris_rotate(R k, const R B[3], R um[3], R gm) {
-    const R kg = k / gm;  // one division for the three components of t
+__device__ __forceinline__ void boris_rotate(R k, const R B[3], R um[3], R g2) {
+    // one division (FP64: none) for the three components of t
+    const R kg = sizeof(R) == 8 ? k * inv_sqrt(g2) : k / sqrt_<R>(g2);
     const R t0 = kg * B[0], t1 = kg * B[1], t2 = kg * B[2];
     const R tt = t0 * t0 + t1 * t1 + t2 * t2;
     const R sc = R(2) / (R(1) + tt);
@@ -200,14 +219,13 @@ __device__ __forceinline__ void boris(R k, const R E[3], const R B[3], R u[3], f
         const double Ed[3] = {double(E[0]), double(E[1]), double(E[2])};
         double umd[3] = {double(u[0]) + kd * Ed[0], double(u[1]) + kd * Ed[1], double(u[2]) + kd * Ed[2]};
         const double Bd[3] = {double(B[0]), double(B[1]), double(B[2])};
-        const double gmd = sqrt(1.0 + umd[0] * umd[0] + umd[1] * umd[1] + umd[2] * umd[2]);
-        boris_rotate<double>(kd, Bd, umd, gmd);
+        boris_rotate<double>(kd, Bd, umd, 1.0 + umd[0] * umd[0] + umd[1] * umd[1] + umd[2] * umd[2]);
         u[0] = R(umd[0] + kd * Ed[0]);
         u[1] = R(umd[1] + kd * Ed[1]);
         u[2] = R(umd[2] + kd * Ed[2]);
         return;
     }
-    boris_rotate<R>(k, B, um, sqrt_<R>(g2));
+    boris_rotate<R>(k, B, um, g2);
     u[0] = um[0] + k * E[0];
     u[1] = um[1] + k * E[1];
     u[2] = um[2] + k * E[2];

@@ -426,8 +426,8 @@ __device__ __forceinline__ void push_particle(const StepArgs<R>& A, R EB[6], con
     else boris<R>(A.kq, EB, EB + 3, u, A.g2_fp64);
     mv.ok = true;
     if (sizeof(R) == 8) {
-        const double gi = 1.0 / sqrt(1.0 + double(u[0]) * double(u[0]) + double(u[1]) * double(u[1]) +
-                                     double(u[2]) * double(u[2]));
+        const double gi = inv_sqrt(1.0 + double(u[0]) * double(u[0]) + double(u[1]) * double(u[1]) +
+                                   double(u[2]) * double(u[2]));
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const double dx = __dmul_rn(__dmul_rn(A.dt, double(u[a])), gi);
