@@ -530,10 +530,18 @@ template <typename R, class LY> __device__ __forceinline__ void zero_jbox(R* sJ)
 // so the lanes of a warp work in neighbouring cells (distinct shared-memory
 // banks).  When the tile's cells split evenly over the warps and the
 // particles are spread evenly enough (no warp's share above 1.25x the mean +
-// 32), warp w owns the w-th group of cells (z-rows of the 4 x 4 x 32 tile)
+// 32) and are many enough, warp w owns the w-th group of cells (z-rows of the
+// 4 x 4 x 32 tile)
 // and its lanes split that group's particles: no two warps then deposit into
 // the same row at the same time.  Otherwise the whole tile is cut into runs
 // of about one cell's worth (or A.run).  Per-warp values.
+// Many enough: three rounds a warp (FP64: one).  Below that the last,
+// part-filled round of every warp weighs more than the rows' conflicts do
+// (order 3, 2 a cell, 64 particles a row: 128^3 1338 us a step by rows, 1299
+// by runs of 2; 32^3 in half-tile slabs at 4 a cell 86.8 against 77.1; at 4 a
+// cell and 128 a row 2039 against 2103).  A work item that has two threads a
+// particle spreads them one a thread (16^3, order 3, 2 a cell, 128 in each of
+// 64 slabs: rows 51.8 us a step, runs of 2 44.6, of 1 42.0).
 struct TileWork {
     int beg, end;                              // the tile's particles
     int wbeg, wend, run, nrun, rstart, rstride;
@@ -550,7 +558,8 @@ __device__ __forceinline__ void plan_tile(const StepArgs<R>& A, int t, TileWork&
     w.wbeg = w.beg;
     w.wend = w.end;
     bool by_warp = false;
-    if (A.run <= 0 && g.cpw % nwarp == 0 && nwarp <= 32) {
+    if (A.run <= 0 && g.cpw % nwarp == 0 && nwarp <= 32 &&
+        cnt >= (sizeof(R) == 8 ? 32 : 96) * nwarp) {
         const int cpw = g.cpw / nwarp;
         const int64_t c0 = (int64_t)t * g.cpw;
         const int gsize =
@@ -571,7 +580,9 @@ __device__ __forceinline__ void plan_tile(const StepArgs<R>& A, int t, TileWork&
         w.rstart = 0;
         w.rstride = 32;
     } else {
-        w.run = A.run > 0 ? A.run : max(1, (cnt + (g.cpw >> 1)) / g.cpw);
+        w.run = A.run > 0                        ? A.run
+                : 2 * cnt <= int(blockDim.x) ? 1
+                                             : max(1, (cnt + (g.cpw >> 1)) / g.cpw);
         w.nrun = (cnt + w.run - 1) / w.run;
         w.rstart = threadIdx.x - lane;
         w.rstride = blockDim.x;
