@@ -1093,10 +1093,12 @@ pic_status pic_step_adjoint(pic_ctx* c, int32_t nsteps, int32_t ckpt_every, doub
             PIC_CUDA(save_state(c, L, state_at(view[j]), meta[view[j]]));
         }
         for (int j = len - 1; j >= 0; --j) {
-            const pic::Snapshot snap = L.view(state_at(view[j]));
+            pic::Snapshot snap = L.view(state_at(view[j]));
+            snap.since_sort = meta[view[j]].since_sort;
             const double t = double(meta[view[j]].step) * c->dt;
             PIC_CUDA(adj_counted(c, 3, [&] { return pic::launch_adj_yee(c, b); }));
-            PIC_CUDA(adj_counted(c, 1, [&] { return pic::launch_adj_particles(c, b, snap, t); }));
+            PIC_CUDA(adj_counted(c, c->prec == PIC_FP32_MIXED && snap.since_sort <= 1 ? 2 : 1,
+                                 [&] { return pic::launch_adj_particles(c, b, snap, t); }));
         }
     }
     if (pic_status s = read_error_word(c)) return s;

@@ -268,6 +268,8 @@ struct Snapshot {
     const void* F[9] = {nullptr};
 };
 // ---- stored states (adjoint checkpoints, autotuner trials) -------------------
+    const int* offsets = nullptr;  // cell offsets of the last sort before the state
+    int since_sort = 0;            // steps since that sort
 // A device allocation freed on scope exit.
 struct DeviceBlock {
     char* p = nullptr;
@@ -311,6 +313,7 @@ struct StateLayout {
         for (int i = 0; i < 9; ++i) s.F[i] = base + part + i * size_t(C) * rs;
         return s;
     }
+        s.offsets = reinterpret_cast<const int*>(base + part + fields);
 };
 
 cudaError_t save_state(pic_ctx* c, const StateLayout& L, char* dst, StateMeta& m);

@@ -414,10 +414,11 @@ template <typename R> struct Moved {
     bool ok;
 };
 
-template <int P, typename R>
+// DRIVE: add the external drive to E_y at the step's own time.
+template <int P, typename R, bool DRIVE = true>
 __device__ __forceinline__ void push_particle(const StepArgs<R>& A, R EB[6], const int cell[3], const R f0[3],
                                               const double xg0[3], R u[3], Moved<R>& mv) {
-    if (A.drive_amp != 0.0) {
+    if (DRIVE && A.drive_amp != 0.0) {
         const double t = double(*A.step) * A.dt;
         const double xp = sizeof(R) == 8 ? xg0[0] : (double(cell[0]) + double(f0[0])) * A.g.d[0];
         EB[1] += R(A.drive_amp * cos(A.drive_k * xp - A.drive_k * t));

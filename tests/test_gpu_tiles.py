@@ -80,3 +80,29 @@ def test_window_on_overhanging_tiles(n, dividing):
     assert rel_l2(a[0], b[0]) < 1e-11
     for k in pic.PARTICLE_KEYS:
         assert np.linalg.norm(a[1][k] - b[1][k]) < 1e-10 * (1 + np.linalg.norm(b[1][k])), k
+
+
+@pytest.mark.parametrize("n,order,tile,moves", [
+    ((9, 7, 11), 1, (0, 0, 0), 0),
+    ((10, 9, 34), 2, (0, 0, 0), 0),
+    ((9, 12, 13), 3, (0, 0, 0), 0),
+    ((8, 8, 64), 3, (0, 0, 0), 0),
+    ((16, 16, 16), 2, (2, 2, 2), 0),
+    ((10, 9, 34), 2, (0, 0, 0), 3),   # three pushes since the sort: particles beyond their slab's box
+])
+def test_fp32_mixed_adjoint_on_tiles_against_fp64(n, order, tile, moves):
+    """The FP32-mixed reverse sweep adds the gather's adjoint by tiles; FP64
+    does so particle by particle.  dL/du within 1e-3, as the 64^3 workload's
+    bound between the two precisions."""
+    out = []
+    for precision in (pic.FP64, pic.FP32_MIXED):
+        c = Case(n, order, 3, 0.4, 229, field_scale=0.05, tile=tile, precision=precision)
+        c.ctx.set_external_drive(0.07, 2 * np.pi / n[0])
+        for _ in range(moves):
+            c.ctx.gather_push()
+        loss, dA, du = c.ctx.step_adjoint(5, 2)
+        out.append((loss, dA, np.asarray(du)))
+    a, b = out
+    assert abs(a[0] - b[0]) < 1e-4 * abs(a[0])
+    assert abs(a[1] - b[1]) < 1e-3 * abs(a[1])
+    assert rel_l2(b[2], a[2]) < 1e-3
