@@ -259,13 +259,13 @@ cudaError_t ensure_tile_order(pic_ctx* c) {
 }
 
 cudaError_t yee_b_half(pic_ctx* c) { return pic::launch_yee_b(c, 0.5 * c->dt); }
+cudaError_t yee_b_last(pic_ctx* c) { return pic::launch_yee_b(c, 0.5 * c->dt, true); }
 
 cudaError_t run_yee(pic_ctx* c) {
     cudaError_t e;
     if ((e = counted(c, "k_yee_b", 1, yee_b_half)) != cudaSuccess) return e;
     if ((e = counted(c, "k_yee_e", 1, pic::launch_yee_e)) != cudaSuccess) return e;
-    if ((e = counted(c, "k_yee_b", 1, yee_b_half)) != cudaSuccess) return e;
-    return counted(c, "k_step_counter", 1, pic::launch_step_counter);
+    return counted(c, "k_yee_b", 1, yee_b_last);
 }
 
 // The particle half and the field half of a step.  With two field sets the

@@ -213,7 +213,8 @@ bool encode_eb_tensor_map(CUtensorMap* map, const void* base, const int n[3], in
                           int prec);
 cudaError_t launch_gather_push_global(pic_ctx* c);
 cudaError_t launch_deposit_global(pic_ctx* c);
-cudaError_t launch_yee_b(pic_ctx* c, double h);
+// count_step: this launch also advances the device step counter
+cudaError_t launch_yee_b(pic_ctx* c, double h, bool count_step = false);
 cudaError_t launch_yee_e(pic_ctx* c);
 // One-pass field update from the current set (E, B) and the other set's J
 // into the other set's E, B, and the step counter advanced (plain Yee, the
@@ -222,7 +223,6 @@ cudaError_t launch_yee_fused(pic_ctx* c);
 cudaError_t configure_yee_fused();
 void swap_field_sets(pic_ctx* c);
 
-cudaError_t launch_step_counter(pic_ctx* c);
 // particles [base, base + n) from arrays that start at particle base
 cudaError_t launch_load_particles(pic_ctx* c, const double* const src[7], int64_t n, int64_t base = 0);
 // particles [p0, p0 + cnt) (current order) into element 0.. of dst / id

@@ -133,8 +133,11 @@ template <typename R> __device__ __forceinline__ void yee_e_at(const YeeArgs<R>&
     yee_e_ijk(Y, c, i, j, k);
 }
 
-// Single-box grids: block x is a z-row (i, j) of the grid, block y a chunk of
-// kBlock cells along it, so no thread divides a 64-bit cell index.
+// Single-box grids: block x is blockDim.y z-rows (i, j) of the grid, block y a
+// chunk of blockDim.x cells along them, so no thread divides a 64-bit cell
+// index.  blockDim.x is the least power of two from 32 to kBlock that covers
+// nz, so that short rows leave few threads idle (96 x 96 x 128, CKC: one row of
+// 256 threads a block took 35 us a B half step).
 struct RowCell {
     int i, j, k;
     int64_t c;
@@ -142,18 +145,18 @@ struct RowCell {
 };
 template <typename R> __device__ __forceinline__ RowCell row_cell(const YeeArgs<R>& Y) {
     RowCell r;
-    const int row = int(blockIdx.x);
+    const int row = int(blockIdx.x) * blockDim.y + threadIdx.y;
     r.i = row / Y.n[1];
     r.j = row - r.i * Y.n[1];
     r.k = int(blockIdx.y) * blockDim.x + threadIdx.x;
-    r.ok = r.k < Y.n[2];
+    r.ok = r.k < Y.n[2] && r.i < Y.n[0];
     r.c = (int64_t)row * Y.n[2] + r.k;
     return r;
 }
 
 template <typename R> __global__ void __launch_bounds__(kBlock) k_yee_b(YeeArgs<R> Y) {
     const RowCell r = row_cell(Y);
-    if (Y.step && r.c == 0) *Y.step += 1;
+    if (Y.step && r.ok && r.c == 0) *Y.step += 1;
     if (r.ok) yee_b_ijk(Y, r.c, r.i, r.j, r.k);
 }
 
@@ -161,7 +164,7 @@ template <typename R> __global__ void __launch_bounds__(kBlock) k_yee_b(YeeArgs<
 // needs must not lower the occupancy of the plain Yee update).
 template <typename R> __global__ void __launch_bounds__(kBlock, 3) k_yee_b_ckc(YeeArgs<R> Y) {
     const RowCell r = row_cell(Y);
-    if (Y.step && r.c == 0) *Y.step += 1;
+    if (Y.step && r.ok && r.c == 0) *Y.step += 1;
     if (r.ok) yee_b_ckc_ijk(Y, r.c, r.i, r.j, r.k);
 }
 
@@ -714,20 +717,28 @@ cudaError_t launch_rekey(int* key, int64_t n, const Geom& from, const Geom& to, 
     return cudaGetLastError();
 }
 
-// z-rows x chunks of kBlock cells along z
+// Threads of a block and blocks of the launch (see row_cell).
+static dim3 yee_block(const pic_ctx* c) {
+    unsigned bz = 32;
+    while (bz < unsigned(kBlock) && bz < unsigned(c->g.n[2])) bz *= 2;
+    return dim3(bz, unsigned(kBlock) / bz);
+}
 static dim3 yee_grid(const pic_ctx* c) {
-    return dim3(unsigned(int64_t(c->g.n[0]) * c->g.n[1]), unsigned((c->g.n[2] + kBlock - 1) / kBlock));
+    const dim3 b = yee_block(c);
+    return dim3(unsigned((int64_t(c->g.n[0]) * c->g.n[1] + b.y - 1) / b.y), unsigned((c->g.n[2] + b.x - 1) / b.x));
 }
 
-cudaError_t launch_yee_b(pic_ctx* c, double h) {
+cudaError_t launch_yee_b(pic_ctx* c, double h, bool count_step) {
     if (c->prec == PIC_FP64) {
         auto Y = make_yee<double>(c, h);
-        if (c->solver) k_yee_b_ckc<double><<<yee_grid(c), kBlock, 0, c->stream>>>(Y);
-        else k_yee_b<double><<<yee_grid(c), kBlock, 0, c->stream>>>(Y);
+        if (count_step) Y.step = c->d_step;
+        if (c->solver) k_yee_b_ckc<double><<<yee_grid(c), yee_block(c), 0, c->stream>>>(Y);
+        else k_yee_b<double><<<yee_grid(c), yee_block(c), 0, c->stream>>>(Y);
     } else {
         auto Y = make_yee<float>(c, h);
-        if (c->solver) k_yee_b_ckc<float><<<yee_grid(c), kBlock, 0, c->stream>>>(Y);
-        else k_yee_b<float><<<yee_grid(c), kBlock, 0, c->stream>>>(Y);
+        if (count_step) Y.step = c->d_step;
+        if (c->solver) k_yee_b_ckc<float><<<yee_grid(c), yee_block(c), 0, c->stream>>>(Y);
+        else k_yee_b<float><<<yee_grid(c), yee_block(c), 0, c->stream>>>(Y);
     }
     return cudaGetLastError();
 }
@@ -783,18 +794,11 @@ cudaError_t configure_yee_fused() {
 cudaError_t launch_yee_e(pic_ctx* c) {
     if (c->prec == PIC_FP64) {
         auto Y = make_yee<double>(c, c->dt);
-        k_yee_e<double><<<yee_grid(c), kBlock, 0, c->stream>>>(Y);
+        k_yee_e<double><<<yee_grid(c), yee_block(c), 0, c->stream>>>(Y);
     } else {
         auto Y = make_yee<float>(c, c->dt);
-        k_yee_e<float><<<yee_grid(c), kBlock, 0, c->stream>>>(Y);
+        k_yee_e<float><<<yee_grid(c), yee_block(c), 0, c->stream>>>(Y);
     }
-    return cudaGetLastError();
-}
-
-__global__ void k_step_counter(long long* s) { *s += 1; }
-
-cudaError_t launch_step_counter(pic_ctx* c) {
-    k_step_counter<<<1, 1, 0, c->stream>>>(c->d_step);
     return cudaGetLastError();
 }
 
@@ -1007,20 +1011,25 @@ cudaError_t launch_continuity(pic_ctx* c, const double* rho0, const double* rho1
 // paper's plasma-acceleration run, Sec. 4.2, in its compensated binomial
 // form): npass passes of (1/4, 1/2, 1/4) along z, then one compensation pass
 // (-npass/4, 1 + npass/2, -npass/4); each pass reads the previous one's output,
-// periodic along z or zero beyond the z ends when z is open.  One CTA per z
-// column of one component, the column ping-ponging between two shared-memory
-// rows of nz values.
+// periodic along z or zero beyond the z ends when z is open.  A group of
+// kBlock / cpb threads takes one z column of one component (consecutive columns
+// are consecutive in memory, across the components too), ping-ponging between
+// two shared-memory rows of nz values.  The launch is short of useful threads
+// and long on barriers when a block holds a single short column (96 x 96 x 128:
+// 135 us at one column a block, floor 8 us), so a block takes as many columns,
+// up to 8 (a warp each), as fit 48 KB.
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void __launch_bounds__(kBlock) k_filter_z(const R* __restrict__ F, R* __restrict__ out, int64_t C, int nz,
-                                                     int npass, int zopen) {
+__global__ void __launch_bounds__(kBlock) k_filter_z(const R* __restrict__ F, R* __restrict__ out, int64_t cols, int nz,
+                                                     int npass, int zopen, int cpb) {
     extern __shared__ __align__(16) unsigned char filt_raw[];
-    R* buf = reinterpret_cast<R*>(filt_raw);  // two rows of nz values
-    const int64_t col = blockIdx.x;           // (i ny + j) of the column
-    const int comp = blockIdx.y;              // 0..5: Ex..Bz
-    const R* src = F + comp * C + col * nz;
-    R* dst = out + comp * C + col * nz;
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) buf[k] = src[k];
+    const int tpc = kBlock / cpb, grp = int(threadIdx.x) / tpc, t0 = int(threadIdx.x) - grp * tpc;
+    R* buf = reinterpret_cast<R*>(filt_raw) + size_t(grp) * 2 * nz;  // the group's two rows
+    const int64_t col = (int64_t)blockIdx.x * cpb + grp;             // component * nx ny + (i ny + j)
+    const bool live = col < cols;
+    const R* src = F + (live ? col : 0) * nz;
+    R* dst = out + (live ? col : 0) * nz;
+    for (int k = t0; k < nz; k += tpc) buf[k] = src[k];
     __syncthreads();
     int cur = 0;
     for (int pass = 0; pass <= npass; ++pass) {
@@ -1028,7 +1037,7 @@ __global__ void __launch_bounds__(kBlock) k_filter_z(const R* __restrict__ F, R*
         const R b = pass < npass ? R(0.5) : R(1.0 + 0.5 * npass);
         const R* in = buf + cur * nz;
         R* o = buf + (1 - cur) * nz;
-        for (int k = threadIdx.x; k < nz; k += blockDim.x) {
+        for (int k = t0; k < nz; k += tpc) {
             const R left = k > 0 ? in[k - 1] : (zopen ? R(0) : in[nz - 1]);
             const R right = k + 1 < nz ? in[k + 1] : (zopen ? R(0) : in[0]);
             o[k] = a * left + b * in[k] + a * right;
@@ -1036,10 +1045,18 @@ __global__ void __launch_bounds__(kBlock) k_filter_z(const R* __restrict__ F, R*
         __syncthreads();
         cur = 1 - cur;
     }
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) dst[k] = buf[cur * nz + k];
+    if (live)
+        for (int k = t0; k < nz; k += tpc) dst[k] = buf[cur * nz + k];
 }
 
-size_t filter_smem_bytes(const pic_ctx* c) { return 2 * size_t(c->g.n[2]) * c->rsize; }
+// Columns a block of the filter takes.
+static int filter_columns(const pic_ctx* c) {
+    int cpb = 1;
+    while (cpb < 8 && 4 * size_t(cpb) * c->g.n[2] * c->rsize <= (48u << 10)) cpb *= 2;
+    return cpb;
+}
+
+size_t filter_smem_bytes(const pic_ctx* c) { return filter_columns(c) * 2 * size_t(c->g.n[2]) * c->rsize; }
 
 cudaError_t configure_filter(const pic_ctx* c) {
     const int bytes = int(filter_smem_bytes(c));
@@ -1050,16 +1067,18 @@ cudaError_t configure_filter(const pic_ctx* c) {
 
 cudaError_t launch_filter(pic_ctx* c) {
     if (c->filter_passes <= 0 || !c->Fg) return cudaSuccess;
-    const dim3 grid(unsigned(int64_t(c->g.n[0]) * c->g.n[1]), 6);
+    const int cpb = filter_columns(c);
+    const int64_t cols = 6 * int64_t(c->g.n[0]) * c->g.n[1];
+    const unsigned grid = unsigned((cols + cpb - 1) / cpb);
     const size_t smem = filter_smem_bytes(c);
     if (c->prec == PIC_FP64)
         k_filter_z<double><<<grid, kBlock, smem, c->stream>>>(static_cast<const double*>(c->F[0]),
-                                                              static_cast<double*>(c->Fg), c->g.C, c->g.n[2],
-                                                              c->filter_passes, c->g.zopen);
+                                                              static_cast<double*>(c->Fg), cols, c->g.n[2],
+                                                              c->filter_passes, c->g.zopen, cpb);
     else
         k_filter_z<float><<<grid, kBlock, smem, c->stream>>>(static_cast<const float*>(c->F[0]),
-                                                             static_cast<float*>(c->Fg), c->g.C, c->g.n[2],
-                                                             c->filter_passes, c->g.zopen);
+                                                             static_cast<float*>(c->Fg), cols, c->g.n[2],
+                                                             c->filter_passes, c->g.zopen, cpb);
     return cudaGetLastError();
 }
 
