@@ -999,6 +999,8 @@ pic_status pic_step(pic_ctx* c, int32_t nsteps) {
                     c->graph = nullptr;
                 }
                 const int cur0 = c->cur, fpar0 = c->fpar;
+                const bool clean0 = c->scan_clean;
+                c->scan_clean = true;  // each replay finds the look-back words clear
                 PIC_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
                 g_capturing = true;
                 g_capture_kernels = 0;
@@ -1008,6 +1010,8 @@ pic_status pic_step(pic_ctx* c, int32_t nsteps) {
                 cudaGraph_t graph = nullptr;
                 cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
                 c->cur = cur0;
+                c->scan_clean = clean0;
+                c->tile_cleared = false;
                 if (c->fpar != fpar0) pic::swap_field_sets(c);  // a capture that stopped after one step
                 if (e1 != cudaSuccess) {
                     if (graph) cudaGraphDestroy(graph);
@@ -1021,7 +1025,9 @@ pic_status pic_step(pic_ctx* c, int32_t nsteps) {
                 c->graph_fpar = fpar0;
                 c->graph_kernels = g_capture_kernels;
             }
+            if (!c->scan_clean) PIC_CUDA(pic::clear_scan_words(c));
             PIC_CUDA(cudaGraphLaunch(c->graph, c->stream));
+            c->scan_clean = true;
             c->launches += c->graph_kernels;
             c->step += 2;
             c->since_sort = 1;

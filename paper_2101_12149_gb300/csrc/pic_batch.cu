@@ -369,8 +369,9 @@ pic_status ensure_graph(pic_batch* b, int nsteps) {
     drop_graph(b);
     const int cur0 = P.cur, since0 = P.since_sort;
     const int64_t step0 = P.step;
-    const bool sorted0 = P.sorted;
+    const bool sorted0 = P.sorted, clean0 = P.scan_clean;
     int64_t kernels = 0;
+    P.scan_clean = false;  // the graph's first scan clears its words itself
     BCUDA(cudaStreamBeginCapture(P.stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e1 = enqueue_steps(b, nsteps, &kernels);
     cudaGraph_t graph = nullptr;
@@ -381,6 +382,7 @@ pic_status ensure_graph(pic_batch* b, int nsteps) {
     P.since_sort = since0;
     P.step = step0;
     P.sorted = sorted0;
+    P.scan_clean = clean0;
     if (e1 != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
         return bcuda(e1, "batch step capture");

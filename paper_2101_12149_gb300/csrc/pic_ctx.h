@@ -130,6 +130,8 @@ struct pic_ctx {
     int* offsets = nullptr;  // exclusive scan of count [K+1]; tile t owns [offsets[t*cpt], offsets[(t+1)*cpt])
     unsigned long long* scan_status = nullptr;  // look-back words + ticket
     int scan_chunks = 0;
+    bool scan_clean = false;    // the look-back words are zero (the last scan's scatter cleared them)
+    bool tile_cleared = false;  // this step's scatter cleared the tile kernel's counters and its current
     bool sorted = false;       // particles are in tile order of the current offsets
     int since_sort = 0;
     // sort bins: 0 = cells (the step's sort); > 0 = runs of 2^sort_shift
@@ -266,10 +268,10 @@ struct Snapshot {
     int* key = nullptr;
     int* id = nullptr;
     const void* F[9] = {nullptr};
-};
-// ---- stored states (adjoint checkpoints, autotuner trials) -------------------
     const int* offsets = nullptr;  // cell offsets of the last sort before the state
     int since_sort = 0;            // steps since that sort
+};
+// ---- stored states (adjoint checkpoints, autotuner trials) -------------------
 // A device allocation freed on scope exit.
 struct DeviceBlock {
     char* p = nullptr;
@@ -311,9 +313,9 @@ struct StateLayout {
         s.key = reinterpret_cast<int*>(base + 7 * per);
         s.id = reinterpret_cast<int*>(base + 7 * per + ints);
         for (int i = 0; i < 9; ++i) s.F[i] = base + part + i * size_t(C) * rs;
+        s.offsets = reinterpret_cast<const int*>(base + part + fields);
         return s;
     }
-        s.offsets = reinterpret_cast<const int*>(base + part + fields);
 };
 
 cudaError_t save_state(pic_ctx* c, const StateLayout& L, char* dst, StateMeta& m);
@@ -356,6 +358,7 @@ cudaError_t configure_batch_kernels();
 // sort (pic_sort.cu)
 cudaError_t launch_hist(pic_ctx* c);
 cudaError_t launch_scan(pic_ctx* c);
+cudaError_t clear_scan_words(pic_ctx* c);
 cudaError_t launch_scatter(pic_ctx* c);
 // the step's sort as a permutation (perm), the particle data left in place
 cudaError_t launch_scatter_perm(pic_ctx* c);

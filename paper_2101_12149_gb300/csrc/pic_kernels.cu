@@ -1216,9 +1216,12 @@ template <typename R> cudaError_t tile_step_dispatch(pic_ctx* c) {
 cudaError_t launch_tile_step(pic_ctx* c) {
     // J is one allocation of three components (see pic_api.cu); the outsider
     // count and the tile queue counter sit after the four error words
-    cudaError_t e = cudaMemsetAsync(c->j_other ? c->Fo[6] : c->F[6], 0, 3 * c->g.C * c->rsize, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->err + 4, 0, 2 * sizeof(unsigned), c->stream);
-    if (e != cudaSuccess) return e;
+    if (!c->tile_cleared) {  // no permutation sort before this step to do it
+        cudaError_t e = cudaMemsetAsync(c->j_other ? c->Fo[6] : c->F[6], 0, 3 * c->g.C * c->rsize, c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->err + 4, 0, 2 * sizeof(unsigned), c->stream);
+        if (e != cudaSuccess) return e;
+    }
+    c->tile_cleared = false;
     return c->prec == PIC_FP64 ? tile_step_dispatch<double>(c) : tile_step_dispatch<float>(c);
 }
 

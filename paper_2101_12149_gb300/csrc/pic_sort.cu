@@ -198,13 +198,45 @@ __global__ void __launch_bounds__(kSortBlock) k_scan(const int* __restrict__ cou
     }
 }
 
+// What the next launches of a step need cleared, done by the scatter on its
+// way (each was a memset of its own: 16^3, order 3, 2 a cell: 42.0 us a step
+// with three of them): the scan's words, read for the last time by the scan
+// before this kernel; the tile kernel's two counters; the current it adds to.
+struct ClearArgs {
+    unsigned long long* status = nullptr;
+    int nstatus = 0;
+    int* counters = nullptr;  // two
+    char* cur = nullptr;      // 4-byte aligned
+    int64_t cur_bytes = 0;    // a multiple of 4
+};
+
+__device__ __forceinline__ void clear_for_step(const ClearArgs& z) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t; i < z.nstatus; i += n) z.status[i] = 0ull;
+    if (z.counters && t < 2) z.counters[t] = 0;
+    if (z.cur_bytes > 0) {
+        // up to three words to a 16-byte boundary, 16 bytes a store, the rest by words
+        const int64_t words = z.cur_bytes >> 2;
+        int64_t head = (int64_t)((16u - unsigned(reinterpret_cast<uintptr_t>(z.cur) & 15u)) & 15u) >> 2;
+        if (head > words) head = words;
+        const int64_t quads = (words - head) >> 2;
+        int* w = reinterpret_cast<int*>(z.cur);
+        if (t < head) w[t] = 0;
+        int4* q = reinterpret_cast<int4*>(w + head);
+        for (int64_t i = t; i < quads; i += n) q[i] = make_int4(0, 0, 0, 0);
+        const int64_t rest = head + 4 * quads;
+        if (t < words - rest) w[rest + t] = 0;
+    }
+}
+
 // `bin` is the array of sort bins: the cell keys themselves (the step's
 // sort) or the bins of pic_sort_particles; the cell key always moves with
 // the particle.
 template <typename E>
 __global__ void __launch_bounds__(kSortBlock) k_scatter(PartBuf src, PartBuf dst, const int* __restrict__ bin,
                                                         int64_t np, const int* offsets, int* count, int64_t C,
-                                                        unsigned* err) {
+                                                        unsigned* err, ClearArgs clear) {
+    clear_for_step(clear);
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int k = -1, key = 0;
     // the particle's data is loaded first: these loads do not depend on the
@@ -249,7 +281,7 @@ constexpr int kPermPerThread = 4;
 // into the other buffer, so the data moves once a step instead of twice.
 __global__ void __launch_bounds__(kSortBlock) k_scatter_perm(const int* __restrict__ bin, int64_t np,
                                                              const int* offsets, int* count, int64_t C, int* perm,
-                                                             unsigned* err) {
+                                                             unsigned* err, ClearArgs clear) {
     // kPermPerThread particles a thread (a block's consecutive particles in
     // kPermPerThread coalesced rows): their slot atomics are in flight at once
     constexpr int U = kPermPerThread;
@@ -286,6 +318,7 @@ __global__ void __launch_bounds__(kSortBlock) k_scatter_perm(const int* __restri
         }
         perm[dest] = int(p0 + u * kSortBlock);
     }
+    clear_for_step(clear);
 }
 
 // SplitMix64 output function (Steele, Lea & Flood 2014): a bijective 64-bit mixer.
@@ -339,32 +372,54 @@ cudaError_t launch_hist(pic_ctx* c) {
     return cudaGetLastError();
 }
 
+cudaError_t clear_scan_words(pic_ctx* c) {
+    return cudaMemsetAsync(c->scan_status, 0, (size_t(c->scan_chunks) + 1) * sizeof(unsigned long long), c->stream);
+}
+
 cudaError_t launch_scan(pic_ctx* c) {
-    cudaError_t e =
-        cudaMemsetAsync(c->scan_status, 0, (size_t(c->scan_chunks) + 1) * sizeof(unsigned long long), c->stream);
-    if (e != cudaSuccess) return e;
+    if (!c->scan_clean) {
+        const cudaError_t e = clear_scan_words(c);
+        if (e != cudaSuccess) return e;
+    }
+    c->scan_clean = false;
     k_scan<<<unsigned(c->scan_chunks), kSortBlock, 0, c->stream>>>(c->count, c->offsets, nbins(c), c->scan_status,
                                                                   c->scan_chunks, c->err);
     return cudaGetLastError();
 }
 
+// The scan's words are cleared by the scatter that follows it.
+static ClearArgs scan_words(const pic_ctx* c) {
+    ClearArgs z;
+    z.status = c->scan_status;
+    z.nstatus = c->scan_chunks + 1;
+    return z;
+}
+
 cudaError_t launch_scatter_perm(pic_ctx* c) {
     if (c->np == 0) return cudaSuccess;
+    ClearArgs z = scan_words(c);
+    z.counters = reinterpret_cast<int*>(c->err + 4);
+    z.cur = static_cast<char*>(c->Fo[0] ? c->Fo[6] : c->F[6]);
+    z.cur_bytes = 3 * c->g.C * int64_t(c->rsize);
+    c->scan_clean = true;
+    c->tile_cleared = true;
     const unsigned nb = unsigned((c->np + kPermPerThread * kSortBlock - 1) / (kPermPerThread * kSortBlock));
     k_scatter_perm<<<nb, kSortBlock, 0, c->stream>>>(bins(c), c->np, c->offsets, c->count, nbins(c), c->perm,
-                                                      c->err);
+                                                      c->err, z);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scatter(pic_ctx* c) {
     if (c->np == 0) return cudaSuccess;
     const unsigned nb = unsigned((c->np + kSortBlock - 1) / kSortBlock);
+    const ClearArgs z = scan_words(c);
+    c->scan_clean = true;
     if (c->prec == PIC_FP64)
         k_scatter<double><<<nb, kSortBlock, 0, c->stream>>>(c->P[c->cur], c->P[1 - c->cur], bins(c), c->np,
-                                                            c->offsets, c->count, nbins(c), c->err);
+                                                            c->offsets, c->count, nbins(c), c->err, z);
     else
         k_scatter<float><<<nb, kSortBlock, 0, c->stream>>>(c->P[c->cur], c->P[1 - c->cur], bins(c), c->np,
-                                                           c->offsets, c->count, nbins(c), c->err);
+                                                           c->offsets, c->count, nbins(c), c->err, z);
     return cudaGetLastError();
 }
 
