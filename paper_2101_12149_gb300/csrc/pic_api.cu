@@ -684,7 +684,7 @@ pic_status pic_init_grid(const pic_grid_desc* desc, void* cuda_stream, pic_ctx**
                 return fail(PIC_ERR_ARG, "tile extents must be powers of two dividing the grid");
             }
     }
-    if (T[0] <= 8 && T[1] <= 8 && T[2] <= 8) c->layout = 0;
+    if (T[0] <= 8 && T[1] <= 8 && T[2] <= 8) c->layout = pic::cube_layout(D.order, D.precision);
     else if (T[0] <= 4 && T[1] <= 4 && T[2] <= 32) c->layout = D.precision == PIC_FP32_MIXED && D.order == 1 ? 2 : 1;
     else {
         delete c;

@@ -111,7 +111,7 @@ struct pic_ctx {
     int* perm = nullptr;     // the step's sort order [cap] (k_scatter_perm)
     bool tile_perm = false;  // the next tile kernel reads the other buffer through perm
     int layout = 0;          // shared-memory layout of the tile kernel: 0 = up to 8x8x8, 1 = 4x4x32,
-                             // 2 = 4x4x32 with a halo of 1 (FP32-mixed, order 1)
+                             // 2, 3 = 4x4x32 and up to 8x8x8 with a halo of 1 (FP32-mixed, order 1)
     int sms = 1;             // streaming multiprocessors of the device (persistent grids)
     // TMA descriptor of E and B (four dimensions z, y, x, component) whose box
     // is one tile's staged E/B block
@@ -208,9 +208,11 @@ cudaError_t launch_tile_step(pic_ctx* c);        // fused gather+push+deposit, t
 cudaError_t configure_tile_kernels(pic_ctx* c);
 // encodes c->tmap_eb where the tile kernel can stage by TMA (sets c->tma)
 void setup_tile_tma(pic_ctx* c);
+// Layout of tiles up to 8x8x8 (pic_ctx::layout).
+inline int cube_layout(int order, int prec) { return order == 1 && prec == PIC_FP32_MIXED ? 3 : 0; }
 // TMA descriptor of the E/B arrays of one box (E and B at `base`, components
-// comp_stride values apart, precision `prec`) for tile layout `layout` (0:
-// 8x8x8, 1: 4x4x32); false (and a zeroed map) where TMA cannot be used
+// comp_stride values apart, precision `prec`) for tile layout `layout`
+// (as pic_ctx::layout); false (and a zeroed map) where TMA cannot be used
 bool encode_eb_tensor_map(CUtensorMap* map, const void* base, const int n[3], int64_t comp_stride, int layout,
                           int prec);
 cudaError_t launch_gather_push_global(pic_ctx* c);
@@ -344,7 +346,7 @@ struct BatchTileLaunch {
     int nboxes = 0;
     const int* outn = nullptr;       // outsider count and list of this order's boxes
     const int* outl = nullptr;
-    int grid = 0;                    // persistent CTAs
+    int sms = 0;                     // streaming multiprocessors (the persistent grid fills them)
 };
 cudaError_t launch_tile_step_batch(int prec, const BatchTileLaunch& L, cudaStream_t s);
 // Yee update of all boxes: yb / ye are YeeArgs<R>[nboxes] with h = dt/2 and

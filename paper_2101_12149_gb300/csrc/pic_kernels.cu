@@ -77,6 +77,9 @@ using LayoutCube = std::conditional_t<sizeof(R) == 4, Layout<8, 8, 8, 24, 24, 2,
                                       Layout<8, 8, 8, 14, 20, 2, 256, 1>>;
 // Order 1, FP32-mixed, 4 x 4 x 32 tiles: halo 1, two CTAs of 256 threads per SM.
 using LayoutRow1 = Layout<4, 4, 32, 40, 40, 1, 256, 2>;
+// The same for tiles up to 8 x 8 x 8: 106 KB a tile with pitches of 20 words
+// (the four z-rows of a warp's cells at banks 0, 20, 8 and 28).
+using LayoutCube1 = Layout<8, 8, 8, 20, 20, 1, 256, 2>;
 
 // Gather of one component from the staged box: `base` points at the first
 // stencil node.
@@ -1201,15 +1204,19 @@ template <typename R, int P, class LY> cudaError_t tile_step_impl(pic_ctx* c) {
 
 template <typename R, class LY> cudaError_t tile_step_order(pic_ctx* c) {
     switch (c->order) {
-    case 1: return tile_step_impl<R, 1, LY>(c);
+    case 1:
+        if constexpr (sizeof(R) == 8) return tile_step_impl<R, 1, LY>(c);
+        return cudaErrorInvalidValue;  // FP32-mixed order 1 has layouts of its own
     case 2: return tile_step_impl<R, 2, LY>(c);
     default: return tile_step_impl<R, 3, LY>(c);
     }
 }
 
 template <typename R> cudaError_t tile_step_dispatch(pic_ctx* c) {
-    if constexpr (sizeof(R) == 4)
+    if constexpr (sizeof(R) == 4) {
         if (c->layout == 2) return tile_step_impl<float, 1, LayoutRow1>(c);
+        if (c->layout == 3) return tile_step_impl<float, 1, LayoutCube1>(c);
+    }
     return c->layout == 1 ? tile_step_order<R, LayoutRow<R>>(c) : tile_step_order<R, LayoutCube<R>>(c);
 }
 
@@ -1239,13 +1246,20 @@ bool encode_eb_tensor_map(CUtensorMap* map, const void* base, const int n[3], in
         return false;
     }
     const bool f64 = prec == PIC_FP64;
-    if (layout == 2 && f64) return false;  // the halo-1 layout is FP32-mixed only
+    if (layout >= 2 && f64) return false;  // the halo-1 layouts are FP32-mixed only
     const cuuint32_t bz = layout == 2 ? LayoutRow1::eY
+                          : layout == 3 ? LayoutCube1::eY
                           : layout == 1 ? (f64 ? LayoutRow<double>::eY : LayoutRow<float>::eY)
                                         : (f64 ? LayoutCube<double>::eY : LayoutCube<float>::eY);
     // x, y extents are the same for both precisions
-    const cuuint32_t by = layout == 2 ? LayoutRow1::EY : layout == 1 ? LayoutRow<float>::EY : LayoutCube<float>::EY;
-    const cuuint32_t bx = layout == 2 ? LayoutRow1::EX : layout == 1 ? LayoutRow<float>::EX : LayoutCube<float>::EX;
+    const cuuint32_t by = layout == 2   ? LayoutRow1::EY
+                          : layout == 3 ? LayoutCube1::EY
+                          : layout == 1 ? LayoutRow<float>::EY
+                                        : LayoutCube<float>::EY;
+    const cuuint32_t bx = layout == 2   ? LayoutRow1::EX
+                          : layout == 3 ? LayoutCube1::EX
+                          : layout == 1 ? LayoutRow<float>::EX
+                                        : LayoutCube<float>::EX;
     const cuuint64_t nz = cuuint64_t(n[2]), ny = cuuint64_t(n[1]), nx = cuuint64_t(n[0]);
     const cuuint64_t dims[4] = {nz, ny, nx, 6};
     const cuuint64_t strides[3] = {nz * rs, ny * nz * rs, cuuint64_t(comp_stride) * rs};  // bytes, dimensions 1..3
@@ -1280,9 +1294,9 @@ cudaError_t configure_tile_kernels(pic_ctx* c) {
     cudaError_t e = cudaSuccess;
 #define PIC_CFG(R, P, LY)                                                              \
     if (e == cudaSuccess) e = set(k_tile_step<P, R, LY>, LY::template smem_bytes<R>());
-    PIC_CFG(float, 1, LayoutRow1)
-    PIC_CFG(float, 1, LayoutRow<float>) PIC_CFG(float, 2, LayoutRow<float>) PIC_CFG(float, 3, LayoutRow<float>)
-    PIC_CFG(float, 1, LayoutCube<float>) PIC_CFG(float, 2, LayoutCube<float>) PIC_CFG(float, 3, LayoutCube<float>)
+    PIC_CFG(float, 1, LayoutRow1) PIC_CFG(float, 1, LayoutCube1)
+    PIC_CFG(float, 2, LayoutRow<float>) PIC_CFG(float, 3, LayoutRow<float>)
+    PIC_CFG(float, 2, LayoutCube<float>) PIC_CFG(float, 3, LayoutCube<float>)
     PIC_CFG(double, 1, LayoutRow<double>) PIC_CFG(double, 2, LayoutRow<double>) PIC_CFG(double, 3, LayoutRow<double>)
     PIC_CFG(double, 1, LayoutCube<double>) PIC_CFG(double, 2, LayoutCube<double>) PIC_CFG(double, 3, LayoutCube<double>)
 #undef PIC_CFG
@@ -1292,9 +1306,7 @@ cudaError_t configure_tile_kernels(pic_ctx* c) {
         case 1:
             if (c->prec == PIC_FP64) (void)(c->layout == 1 ? tile_grid<double, 1, LayoutRow<double>>(c)
                                                            : tile_grid<double, 1, LayoutCube<double>>(c));
-            else (void)(c->layout == 2   ? tile_grid<float, 1, LayoutRow1>(c)
-                        : c->layout == 1 ? tile_grid<float, 1, LayoutRow<float>>(c)
-                                         : tile_grid<float, 1, LayoutCube<float>>(c));
+            else (void)(c->layout == 2 ? tile_grid<float, 1, LayoutRow1>(c) : tile_grid<float, 1, LayoutCube1>(c));
             break;
         case 2:
             if (c->prec == PIC_FP64) (void)(c->layout == 1 ? tile_grid<double, 2, LayoutRow<double>>(c)
@@ -1313,11 +1325,14 @@ cudaError_t configure_tile_kernels(pic_ctx* c) {
 }
 
 // ---- batch of boxes ----------------------------------------------------------
+template <int P, typename R>
+using BatchLayout = std::conditional_t<P == 1 && sizeof(R) == 4, LayoutCube1, LayoutCube<R>>;
+
 template <typename R, int P> cudaError_t tile_batch_impl(const BatchTileLaunch& L, cudaStream_t s) {
-    using LY = LayoutCube<R>;
+    using LY = BatchLayout<P, R>;
     if (L.nitems <= 0) return cudaSuccess;
     const size_t smem = LY::template smem_bytes<R>();
-    const int grid = L.grid < L.nitems ? L.grid : L.nitems;
+    const int ctas = L.sms * LY::kMinBlocks, grid = ctas < L.nitems ? ctas : L.nitems;
     k_tile_step_batch<P, R, LY><<<unsigned(grid), LY::kThreads, smem, s>>>(
         static_cast<const StepArgs<R>*>(L.boxes), L.items, L.nitems, L.queue);
     cudaError_t e = cudaGetLastError();
@@ -1348,7 +1363,8 @@ cudaError_t configure_batch_kernels() {
     };
     cudaError_t e = cudaSuccess;
 #define PIC_CFG(R, P) \
-    if (e == cudaSuccess) e = set(k_tile_step_batch<P, R, LayoutCube<R>>, LayoutCube<R>::template smem_bytes<R>());
+    if (e == cudaSuccess)   \
+        e = set(k_tile_step_batch<P, R, BatchLayout<P, R>>, BatchLayout<P, R>::template smem_bytes<R>());
     PIC_CFG(float, 1) PIC_CFG(float, 2) PIC_CFG(float, 3) PIC_CFG(double, 1) PIC_CFG(double, 2) PIC_CFG(double, 3)
 #undef PIC_CFG
     return e;
