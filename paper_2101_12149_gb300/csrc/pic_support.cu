@@ -464,7 +464,20 @@ __global__ void k_load(StepArgs<R> A, const double* x, const double* y, const do
     if (!ok) raise_error(A.err, ERRBIT_PARTICLE);
 }
 
-// Particles [p0, p0 + cnt) into element 0.. of the destination arrays.
+// double(v), by moving the bits: exact, and free of the FP64 pipe, on which a
+// conversion takes a warp 16 cycles.  Subnormals, infinities and NaN convert.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)  // normal: rebias the exponent by 1023 - 127
+        return __hiloint2double(int((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), int(b << 29));
+    return m == 0u ? __hiloint2double(int(b), 0) : double(v);
+}
+
+// Particles [p0, p0 + cnt) into element 0.. of the destination arrays.  For
+// FP32-mixed the FP64 pipe bounded it (25 operations a particle: conversions,
+// products and the wrap's compares); six are left where the cells are unit
+// cubes, as integer compares find the positions that round up to the end.
 template <typename R>
 __global__ void k_store(StepArgs<R> A, int64_t p0, int64_t cnt, double* x, double* y, double* z, double* ux,
                         double* uy, double* uz, double* w, const int* idsrc, int32_t* id) {
@@ -478,18 +491,29 @@ __global__ void k_store(StepArgs<R> A, int64_t p0, int64_t cnt, double* x, doubl
     if (sizeof(R) == 4) cell_of(g, A.key[p], cell[0], cell[1], cell[2]);
     for (int a = 0; a < 3; ++a) {
         if (xs[a]) {
-            double v = sizeof(R) == 8 ? double(A.pa[a][p]) : (double(cell[a]) + double(A.pa[a][p])) * g.d[a];
-            xs[a][i] = wrap_pos(v, g.L[a]);
+            double v;
+            if (sizeof(R) == 8) {
+                v = wrap_pos(double(A.pa[a][p]), g.L[a]);
+            } else {
+                // 2^52 + cell by its bits, less 2^52: double(cell), 0 <= cell < 2^31
+                v = (__hiloint2double(0x43300000, cell[a]) - 4503599627370496.0) + widen(A.pa[a][p]);
+                if (g.d[a] != 1.0) v *= g.d[a];
+                const long long b = __double_as_longlong(v);
+                if (b < 0 || b >= __double_as_longlong(g.L[a])) v = wrap_pos(v, g.L[a]);
+            }
+            xs[a][i] = v;
         }
-        if (us[a]) us[a][i] = double(A.pa[3 + a][p]);
+        if (us[a]) us[a][i] = widen(A.pa[3 + a][p]);
     }
-    if (w) w[i] = double(A.pa[6][p]);
+    if (w) w[i] = widen(A.pa[6][p]);
     if (id) id[i] = idsrc[p];
 }
 
 template <typename S, typename D> __global__ void k_convert(const S* src, D* dst, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = D(src[i]);
+    if (i >= n) return;
+    if constexpr (sizeof(S) == 4) dst[i] = widen(src[i]);
+    else dst[i] = D(src[i]);
 }
 
 // out[0] += sum |F|^2 / 2 over Ex..Bz (times dV on the host), out[1] kinetic,
@@ -588,19 +612,29 @@ __global__ void k_diag_divb(const R* Bx, const R* By, const R* Bz, int nx, int n
 // moving window (z open)
 // ---------------------------------------------------------------------------
 // F(i,j,k) <- F(i,j,k+1), F(i,j,nz-1) <- 0 in place: one warp per z column
-// walks it in chunks of 32 (each element is read before it is overwritten:
-// in the same chunk by the warp's load, or by the previous chunk's).
+// walks it in runs of kShiftRun chunks of 32, a run's loads all in flight
+// before its first store (each element is read before it is overwritten: by
+// its own run's loads or by the run before).
+constexpr int kShiftRun = 8;
 template <typename R>
 __global__ void __launch_bounds__(kBlock) k_shift_fields(R* F0, int64_t C, int nz, int64_t columns) {
     const int64_t col = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (col >= columns) return;
     R* f = F0 + (int64_t)blockIdx.y * C + col * nz;
-    for (int k0 = 0; k0 < nz; k0 += 32) {
-        const int k = k0 + lane;
-        const R v = k + 1 < nz ? f[k + 1] : R(0);
+    for (int k0 = lane; k0 - lane < nz; k0 += 32 * kShiftRun) {
+        R v[kShiftRun];
+#pragma unroll
+        for (int r = 0; r < kShiftRun; ++r) {
+            const int k = k0 + 32 * r;
+            v[r] = k + 1 < nz ? f[k + 1] : R(0);
+        }
         __syncwarp();
-        if (k < nz) f[k] = v;
+#pragma unroll
+        for (int r = 0; r < kShiftRun; ++r) {
+            const int k = k0 + 32 * r;
+            if (k < nz) f[k] = v[r];
+        }
         __syncwarp();
     }
 }
