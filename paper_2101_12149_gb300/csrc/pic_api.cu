@@ -288,7 +288,7 @@ cudaError_t run_tile_and_fields(pic_ctx* c, bool count_next = false) {
     c->count_into = false;
     if (e != cudaSuccess) return e;
     if (!c->Fo[0]) return run_yee(c);
-    if ((e = counted(c, "k_yee_fused", 1, pic::launch_yee_fused)) != cudaSuccess) return e;
+    if ((e = counted(c, "k_yee_fused", c->prec == PIC_FP64 ? 3 : 1, pic::launch_yee_fused)) != cudaSuccess) return e;
     pic::swap_field_sets(c);
     return cudaSuccess;
 }

@@ -215,6 +215,8 @@ template <typename R> void fill_args(const pic_batch* b, std::vector<char>& host
             Y.J[d] = reinterpret_cast<const R*>(static_cast<char*>(P.F[6 + d]) + B.cbase * sizeof(R));
             Y.n[d] = B.n[d];
             Y.inv[d] = R(1.0 / B.d[d]);
+            Y.Eo[d] = Y.E[d];
+            Y.Bo[d] = Y.B[d];
         }
         Y.step = nullptr;
         Y.zopen = 0;

@@ -185,11 +185,14 @@ template <typename R> StepArgs<R> make_args_perm(pic_ctx* c, int src, int dst, c
     return a;
 }
 
-// Arguments of the Yee kernels: E, B, J of one box, its extents, inverse
-// cell sizes and the time step h of the update (dt/2 for a B half step).
+// Arguments of the Yee kernels: E, B, J of one box, where the updated E or B
+// goes (the same arrays or another field set's), its extents, inverse cell
+// sizes and the time step h of the update (dt/2 for a B half step).
 template <typename R> struct YeeArgs {
     R* E[3];
     R* B[3];
+    R* Eo[3];
+    R* Bo[3];
     const R* J[3];
     int n[3];
     R inv[3];
