@@ -180,6 +180,8 @@ struct pic_ctx {
     int inj_ppc = 0;
     double inj_n0 = 0.0, inj_ramp_start = 0.0, inj_ramp_length = 0.0;
     int64_t next_id = 0;
+    int zshift = 0;         // the step under way moves the window one cell: its tile kernel and field update write shifted
+    bool j_unshifted = false;  // ... and left its current where it was deposited
 
     cudaGraphExec_t graph = nullptr;
     int graph_cur = 0;
@@ -247,6 +249,8 @@ cudaError_t launch_continuity(pic_ctx* c, const double* rho0, const double* rho1
 // moving window: move fields and particles down one cell along z (particles
 // below z = 0 die), then fill the front slab with plasma at slots [np, np + nx*ny*ppc)
 cudaError_t launch_window_shift(pic_ctx* c);
+// field components [first, first + count) of the current set down one cell along z
+cudaError_t launch_shift_fields(pic_ctx* c, int first, int count);
 cudaError_t launch_inject(pic_ctx* c);
 // bins of pic_sort_particles (sort_shift != 0) into sortbin (pic_sort.cu)
 cudaError_t launch_bin_keys(pic_ctx* c);

@@ -92,6 +92,7 @@ template <typename R> struct StepArgs {
     float vscale;       // FP32-mixed fixed-point scale of the deposit (largest power of two <= 2^30 / max|coef|)
     float inv_vscale;   // 1 / vscale (a power of two: exact)
     int64_t np;
+    int zshift;  // z open: 1 moves every stored particle down one cell along z (the window's shift)
     const CUtensorMap* tmap;  // batch of boxes: the box's E/B TMA descriptor in global memory, or null
     float g2_fp64;            // FP32-mixed: gamma^2 above which the push's rotation runs in FP64
     // Sorted-order step: the tile kernel reads the particle perm[s] of the
@@ -157,6 +158,7 @@ template <typename R> StepArgs<R> make_args(pic_ctx* c) {
         a.inv_vscale = float(std::ldexp(1.0, 1 - e));
     }
     a.np = c->np;
+    a.zshift = c->zshift;
     a.tmap = nullptr;
     a.g2_fp64 = std::isfinite(c->gamma_fp64) ? float(c->gamma_fp64 * c->gamma_fp64) : INFINITY;
     a.perm = nullptr;
@@ -550,7 +552,8 @@ __device__ __forceinline__ void decode_particle(const StepArgs<R>& A, const RawP
 }
 
 // Store the moved particle in place: momentum, wrapped position, new cell key.
-// With z open, a particle whose new z is outside [0, Lz) gets the removed key.
+// With z open, a particle whose new z is outside [0, Lz) gets the removed key;
+// so does one that the window's shift, when the step has one, moves below 0.
 template <typename R>
 __device__ __forceinline__ void store_particle(const StepArgs<R>& A, int p, const int cell[3], const Moved<R>& mv) {
     const Geom& g = A.g;
@@ -562,7 +565,13 @@ __device__ __forceinline__ void store_particle(const StepArgs<R>& A, int p, cons
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             double xw = mv.xg1[a];
-            if (a == 2 && g.zopen) gone = !(xw >= 0.0 && xw < g.L[2]);
+            if (a == 2 && g.zopen) {
+                gone = !(xw >= 0.0 && xw < g.L[2]);
+                if (A.zshift && !gone) {
+                    xw -= g.d[2];
+                    gone = !(xw >= 0.0);
+                }
+            }
             else xw = wrap_pos(xw, g.L[a]);
             A.pa[a][p] = R(xw);
             double f;
@@ -577,8 +586,8 @@ __device__ __forceinline__ void store_particle(const StepArgs<R>& A, int p, cons
                 nf = float(mv.f1[2]) - fl;
                 int cz = cell[2] + int(fl);
                 if (nf >= 1.0f) nf -= 1.0f, cz += 1;
-                gone = unsigned(cz) >= unsigned(g.n[2]);
-                nc[2] = gone ? 0 : cz;
+                gone = unsigned(cz) >= unsigned(g.n[2]) || cz < A.zshift;
+                nc[2] = gone ? 0 : cz - A.zshift;
             } else {
                 renormalise(float(mv.f1[a]), cell[a], g.n[a], nc[a], nf);
             }

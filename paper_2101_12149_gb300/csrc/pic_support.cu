@@ -221,6 +221,7 @@ template <typename R> struct YeeFusedArgs {
     R dt;
     long long* step;
     int zopen;
+    int zshift;  // 1: E and B are written one cell down along z, the top plane zero (the window's shift)
 };
 
 // One element copied global -> shared without passing through registers
@@ -356,13 +357,20 @@ template <typename R> __global__ void __launch_bounds__(kYThreads) k_yee_fused(Y
             const R dEy_dx = (Ec[kEP + ce] - ey) * Y.inv[0];
             const R dEx_dy = (Ep[jp] - ex) * Y.inv[1];
             // the tile's own cells need no wrap: row j0 + warp, z = zj
-            const int64_t g = int64_t(i) * sx + int64_t(j0 + warp) * Y.n[2] + zj;
-            Y.Bo[0][g] = B0[cb] - h * (dEz_dy - dEy_dz);
-            Y.Bo[1][g] = B0[kBP + cb] - h * (dEx_dz - dEz_dx);
-            Y.Bo[2][g] = B0[2 * kBP + cb] - h * (dEy_dx - dEx_dy);
-            Y.Eo[0][g] = ex;
-            Y.Eo[1][g] = ey;
-            Y.Eo[2][g] = ez;
+            const int64_t row = int64_t(i) * sx + int64_t(j0 + warp) * Y.n[2];
+            const int64_t g = row + zj - Y.zshift;
+            if (Y.zshift && zj + 1 == Y.n[2]) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) Y.Bo[c][row + zj] = Y.Eo[c][row + zj] = R(0);
+            }
+            if (zj >= Y.zshift) {
+                Y.Bo[0][g] = B0[cb] - h * (dEz_dy - dEy_dz);
+                Y.Bo[1][g] = B0[kBP + cb] - h * (dEx_dz - dEz_dx);
+                Y.Bo[2][g] = B0[2 * kBP + cb] - h * (dEy_dx - dEx_dy);
+                Y.Eo[0][g] = ex;
+                Y.Eo[1][g] = ey;
+                Y.Eo[2][g] = ez;
+            }
         }
         // rotate the rings
         const int ep = eP;
@@ -711,7 +719,9 @@ template <typename R> __global__ void __launch_bounds__(kBlock) k_inject(StepArg
     A.pa[4][p] = R(0);
     A.pa[5][p] = R(0);
     A.pa[6][p] = R(dens * g.d[0] * g.d[1] * g.d[2] / I.ppc);
-    A.key[p] = dens > 0.0 ? key_of(g, i, j, k) : dead_key(g);
+    const int key = dens > 0.0 ? key_of(g, i, j, k) : dead_key(g);
+    A.key[p] = key;
+    if (A.cnext) atomicAdd(A.cnext + key, 1);
     id[p] = int(I.first_id + t);
 }
 
@@ -805,6 +815,7 @@ template <typename R> cudaError_t yee_fused_impl(pic_ctx* c) {
     Y.dt = R(c->dt);
     Y.step = c->d_step;
     Y.zopen = c->g.zopen;
+    Y.zshift = c->zshift;
     const int64_t blocks = int64_t(Y.nt[0]) * Y.nt[1] * Y.nt[2];
     k_yee_fused<R><<<unsigned(blocks), kYThreads, yee_fused_smem<R>(), c->stream>>>(Y);
     return cudaGetLastError();
@@ -1136,11 +1147,20 @@ cudaError_t launch_filter(pic_ctx* c) {
     return cudaGetLastError();
 }
 
-template <typename R> cudaError_t window_shift_impl(pic_ctx* c) {
+cudaError_t launch_shift_fields(pic_ctx* c, int first, int count) {
     const int64_t columns = int64_t(c->g.n[0]) * c->g.n[1];
-    const dim3 grid(unsigned((columns * 32 + kBlock - 1) / kBlock), 9);
-    k_shift_fields<R><<<grid, kBlock, 0, c->stream>>>(static_cast<R*>(c->F[0]), c->g.C, c->g.n[2], columns);
-    cudaError_t e = cudaGetLastError();
+    const dim3 grid(unsigned((columns * 32 + kBlock - 1) / kBlock), unsigned(count));
+    if (c->prec == PIC_FP64)
+        k_shift_fields<double><<<grid, kBlock, 0, c->stream>>>(static_cast<double*>(c->F[first]), c->g.C, c->g.n[2],
+                                                               columns);
+    else
+        k_shift_fields<float><<<grid, kBlock, 0, c->stream>>>(static_cast<float*>(c->F[first]), c->g.C, c->g.n[2],
+                                                              columns);
+    return cudaGetLastError();
+}
+
+template <typename R> cudaError_t window_shift_impl(pic_ctx* c) {
+    const cudaError_t e = launch_shift_fields(c, 0, 9);
     if (e != cudaSuccess || c->np == 0) return e;
     k_shift_particles<R><<<blocks_for(c->np), kBlock, 0, c->stream>>>(make_args<R>(c));
     return cudaGetLastError();
