@@ -97,25 +97,15 @@ template <typename R> struct Shape<2, R> {
 
 template <typename R> struct Shape<3, R> {
     __device__ __forceinline__ static void weights(R f, int& first, R w[4]) {
+        // the pieces are mirror images in f and g: 13 operations (the FP64 pipe
+        // bounds that path), and the second inner weight rounds as the first
         first = -1;
         const R sixth = R(1) / R(6);
-        const R f2 = f * f, g = R(1) - f;
-        if constexpr (sizeof(R) == 8) {
-            // the pieces are mirror images in f and g: 11 operations on the FP64
-            // pipe, which bounds that path, against 15 (in FP32 the rounding of
-            // 2/3 would raise the bias of the weights' sum from 3.0e-8 to 4.2e-8)
-            const R g2 = g * g, two_thirds = R(2) / R(3);
-            w[0] = g2 * g * sixth;
-            w[1] = two_thirds + f2 * (R(0.5) * f - R(1));
-            w[2] = two_thirds + g2 * (R(0.5) * g - R(1));
-            w[3] = f2 * f * sixth;
-        } else {
-            const R f3 = f2 * f;
-            w[0] = g * g * g * sixth;
-            w[1] = (R(4) - R(6) * f2 + R(3) * f3) * sixth;
-            w[2] = (R(1) + R(3) * f + R(3) * f2 - R(3) * f3) * sixth;
-            w[3] = f3 * sixth;
-        }
+        const R f2 = f * f, g = R(1) - f, g2 = g * g;
+        w[0] = g2 * g * sixth;
+        w[1] = (R(4) + f2 * (R(3) * f - R(6))) * sixth;
+        w[2] = (R(4) + g2 * (R(3) * g - R(6))) * sixth;
+        w[3] = f2 * f * sixth;
     }
 };
 
