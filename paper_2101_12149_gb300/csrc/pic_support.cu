@@ -136,8 +136,8 @@ template <typename R> __device__ __forceinline__ void yee_e_at(const YeeArgs<R>&
 // Single-box grids: block x is blockDim.y z-rows (i, j) of the grid, block y a
 // chunk of blockDim.x cells along them, so no thread divides a 64-bit cell
 // index.  blockDim.x is the least power of two from 32 to kBlock that covers
-// nz, so that short rows leave few threads idle (96 x 96 x 128, CKC: one row of
-// 256 threads a block took 35 us a B half step).
+// nz, so that short rows leave few threads idle (96 x 96 x 128, CKC: a B half
+// step took 35 us at one row of 256 threads a block, 27 us now).
 struct RowCell {
     int i, j, k;
     int64_t c;
@@ -825,7 +825,7 @@ template <typename R> cudaError_t yee_fused_impl(pic_ctx* c) {
 // set, E into the other set, the second B half step there in place).  The
 // one-pass kernel computes B' and E' again in its tiles' and x-chunks' halos,
 // and the FP64 pipe, not the memory, bounds either: 57 operations a cell here
-// (32^3: 29 -> 14 us, 64^3: 72 -> 40 us).
+// (32^3: 29 -> 16 us, 64^3: 72 -> 41, 128^3: 328 -> 210).
 static cudaError_t yee_passes_f64(pic_ctx* c) {
     const dim3 grid = yee_grid(c), block = yee_block(c);
     auto Y = make_yee<double>(c, 0.5 * c->dt);
@@ -1081,7 +1081,7 @@ cudaError_t launch_continuity(pic_ctx* c, const double* rho0, const double* rho1
 // are consecutive in memory, across the components too), ping-ponging between
 // two shared-memory rows of nz values.  The launch is short of useful threads
 // and long on barriers when a block holds a single short column (96 x 96 x 128:
-// 135 us at one column a block, floor 8 us), so a block takes as many columns,
+// 135 us at one column a block, 35 us now, floor 8 us), so a block takes as many columns,
 // up to 8 (a warp each), as fit 48 KB.
 // ---------------------------------------------------------------------------
 template <typename R>
