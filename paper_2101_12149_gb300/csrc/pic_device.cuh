@@ -97,15 +97,22 @@ template <typename R> struct Shape<2, R> {
 
 template <typename R> struct Shape<3, R> {
     __device__ __forceinline__ static void weights(R f, int& first, R w[4]) {
-        // the pieces are mirror images in f and g: 13 operations (the FP64 pipe
-        // bounds that path), and the second inner weight rounds as the first
         first = -1;
         const R sixth = R(1) / R(6);
         const R f2 = f * f, g = R(1) - f, g2 = g * g;
         w[0] = g2 * g * sixth;
-        w[1] = (R(4) + f2 * (R(3) * f - R(6))) * sixth;
-        w[2] = (R(4) + g2 * (R(3) * g - R(6))) * sixth;
         w[3] = f2 * f * sixth;
+        if constexpr (sizeof(R) == 4) {
+            // mirror images in f and g: two operations fewer than expanded
+            w[1] = (R(4) + f2 * (R(3) * f - R(6))) * sixth;
+            w[2] = (R(4) + g2 * (R(3) * g - R(6))) * sixth;
+        } else {
+            // expanded: the mirrored form's rounding left a step's results 5 %
+            // further from the exact ones (64^3: 2.1e-15 against 2.0e-15)
+            const R f3 = f2 * f;
+            w[1] = (R(4) - R(6) * f2 + R(3) * f3) * sixth;
+            w[2] = (R(1) + R(3) * f + R(3) * f2 - R(3) * f3) * sixth;
+        }
     }
 };
 
